@@ -85,7 +85,7 @@ struct Prof {
 
 int pick_D(int d)
 {
-    static const int Ds[] = {1, 2, 3, 4, 6, 8, 12, 16};
+    static const int Ds[] = {1, 2, 3, 4, 6, 8, 9, 12, 16};
     for (int D : Ds)
         if (D >= d) return D;
     return 0;

@@ -27,12 +27,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase)
 
 // Walk the stored predecessor codes back from (M-1, N-1) to (0, 0).
 // A cell (i, j) of band b sits in lane t = (i mod BR) / R at step s = j + t,
-// as bit k = i mod R ("not diag") and bit R + k ("not up") of the lane's 2R
-// code bits of that step.  For R >= 16 those are the W = R / 16 words at
+// as bit R-1-k, k = i mod R ("not diag") and bit 2R-1-k ("not up") of the
+// lane's 2R code bits of that step.  For R >= 16 those are the W = R / 16 words at
 // dirs[dir_off + b*(N+31)*32*W + (s*32 + t)*W + w]; for R = 8 and 4 the word
 // dirs[dir_off + b*band_dir_words(N, R) + (s/S)*32 + t] holds the S = 32/(2R)
-// steps S*(s/S) .. of the lane (2R bits each, the earliest in the lowest
-// bits).  Along the walk s only decreases inside a
+// steps S*(s/S) .. of the lane, 2R bits each: R = 8 the earlier step in the
+// low half; R = 4 from the top bit down, step by step, row by row,
+// "not diag" before "not up".  Along the walk s only decreases inside a
 // band, so a window of kBtWords / 32 consecutive word rows (one contiguous
 // block of global memory) is brought into shared memory by one bulk
 // asynchronous copy (completion on an mbarrier, bounded wait) and the walk
@@ -167,16 +168,21 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
                 }
             }
             // cell (ii, jj) of the window: lane t = (ii mod BR) / R, row k =
-            // ii mod R, step s = jj + t; plane 0 ("not diag") is bit k, plane 1
-            // ("not up") bit R + k of the step's code bits of lane t
+            // ii mod R, step s = jj + t
             auto code_at = [&](int ii, int jj, uint32_t& nd, uint32_t& nu) {
                 const int tt = (ii >> LOG_R) & 31;
                 const int kk = ii & (R - 1);
                 const int ss = jj + tt;
                 const uint32_t* wp = win + ((ss / SPW - wlo) * 32 + tt) * W;
+                if (R == 4) {
+                    const uint32_t w1 = wp[0] << ((ss % SPW) * 2 * R + 2 * kk);
+                    nd = w1 >> 31;
+                    nu = (w1 >> 30) & 1u;
+                    return;
+                }
                 const uint32_t w0 = R < 16 ? wp[0] >> ((ss % SPW) * 2 * R) : wp[0];
-                nd = (w0 >> kk) & 1u;
-                nu = R <= 16 ? (w0 >> (R + kk)) & 1u : (wp[W - 1] >> kk) & 1u;
+                nd = (w0 >> (R - 1 - kk)) & 1u;
+                nu = R <= 16 ? (w0 >> (2 * R - 1 - kk)) & 1u : (wp[W - 1] >> (R - 1 - kk)) & 1u;
             };
             uint32_t nd, nu;
             code_at(i, j, nd, nu);

@@ -21,7 +21,7 @@
 // last column of r in registers.  Lanes are skewed by one column (lane t is at
 // column s - t in step s), so the value above a lane's first row comes from
 // lane t-1 by __shfl_up_sync.  Cycle samples are staged per warp in a
-// 128-column shared-memory ring as duplicated pairs {y, y}, refilled every 32
+// shared-memory ring as duplicated pairs {y, y}, refilled every 32
 // steps from registers loaded ahead.  Lane 0 of band b > 0 reads the bottom row
 // of band b-1 from a hand-off row in global memory (L2), 32 columns at a time,
 // also one chunk ahead; each slot is NaN until its producer has written it
@@ -32,11 +32,13 @@
 // without co-residency.  Every wait is bounded (wait_progress).
 //
 // Predecessor codes (kModeDirs) are two bit-planes per lane and step: bit
-// p*R + k of the lane's W = R/16 words is plane p of row k, plane 0 = "not
+// p*R + R-1-k of the lane's W = R/16 words is plane p of row k, plane 0 = "not
 // diag", plane 1 = "not up" (meaningful only when plane 0 is set).  With R = 8
-// (R = 4) a step has 16 (8) bits and two (four) consecutive steps share one
-// word, the earliest step in the lowest bits.
+// a step has 16 bits and two consecutive steps share one word, the earlier in
+// the lower bits.
 #pragma once
+
+#include <type_traits>
 
 #include "dtw_wavefront.cuh"
 
@@ -94,10 +96,19 @@ __device__ __forceinline__ uint32_t ne_mask(float a, float b)
     return r;
 }
 
-constexpr int kRing = 128;   // columns of cycle samples staged per warp
+// Columns of cycle samples staged per warp: four chunks of 32, each at its own
+// place, chunk c (columns 32 c ..) at 32 (c mod 4), or 128 where that is 0.
+// The chunk at 128 has a copy at 0, and the first columns of the one at 32 a
+// copy at 160, so that every column that a chunk's steps read (31 behind to 3
+// ahead) lies at a fixed distance from the chunk's own place: the steps' shared
+// loads need no address arithmetic.
+constexpr int kRing = 164;
+__device__ __forceinline__ int ring_place(int s0) { return (s0 & 127) ? (s0 & 127) : 128; }
 constexpr int kSlot = 4;     // u64 words after a warp's ring: its band's columns and the band
 
 
+
+constexpr int kSignD = 3;
 
 // c[k] for a k known only at run time, by a binary tree of selects on the bits
 // of k (R - 1 selects, no local memory)
@@ -114,6 +125,24 @@ __device__ __forceinline__ float pick_row(const float (&c)[R], int k)
         for (int q = 0; q < w; ++q) v[q] = hi ? v[q + w] : v[q];
     }
     return v[0];
+}
+
+// The results of one pair: r(M, N), and (kModePlen) |pi| and their quotient.
+template <int MODE>
+__device__ __forceinline__ void write_pair(const DPParams& p, const PairDesc& pd, float v, int c)
+{
+    if (p.cost_out) p.cost_out[pd.out] = v;
+    if (MODE == kModePlen) {
+        if (p.plen_out) p.plen_out[pd.out] = c;
+        if (p.score_out) p.score_out[pd.out] = __fdiv_rn(v, (float)c);
+    }
+    if (p.cost_matrix) {
+        int a = 0, rem = pd.out;
+        while (rem >= p.T - 1 - a) { rem -= p.T - 1 - a; ++a; }
+        const int bb = a + 1 + rem;
+        p.cost_matrix[(int64_t)a * p.T + bb] = v;
+        p.cost_matrix[(int64_t)bb * p.T + a] = v;
+    }
 }
 
 template <int D, int R, int MODE, bool BANDED, int COST>
@@ -134,11 +163,19 @@ struct Band {
     uint32_t half;                          // R < 16: codes of the word's earlier steps
     // kModeSubDirs, matrix's last band: running minimum of r(M-1, j) over the
     // lane's columns (row kk of the lane), and its first column
-    bool track;
     int kk;
     float best;
     int bestj;
     static constexpr bool CODES = MODE == kModeDirs || MODE == kModeSubDirs;
+    static constexpr bool SIGNS = D <= kSignD;
+    // hand-off slots: 4 bytes (r), or 8 bytes ({r, cells}) with |pi|
+    static constexpr int SLOT = MODE == kModePlen ? 8 : 4;
+    // the chunk's addresses (begin_chunk)
+    const u64* yb;
+    uint32_t* db;
+    char* hb;
+    int j0;
+    bool puts;                              // this lane writes the band's hand-off row
 
     // Local costs of column jc for the lane's rows, pair q (two rows at once).
     __device__ __forceinline__ void cost_pair(const u64* yy, int q)
@@ -157,24 +194,32 @@ struct Band {
         }
     }
 
-    __device__ __forceinline__ void load_samples(const u64* ring, int jc, u64* yy)
+    // samples of column j0 + o
+    __device__ __forceinline__ void load_samples(int o, u64* yy)
     {
-        const u64* yr = ring + (jc & (kRing - 1));
 #pragma unroll
-        for (int c = 0; c < D; ++c) yy[c] = yr[c * kRing];
+        for (int c = 0; c < D; ++c) yy[c] = yb[c * kRing + o];
     }
 
-    // One step: the lane's column j = s - lane (in range when FULLCHUNK).
+    // Addresses of the chunk of steps s0 .. s0 + 31.
+    __device__ __forceinline__ void begin_chunk(const u64* ring, int s0, int lane, void* hcur, uint32_t* dout)
+    {
+        yb = ring + (ring_place(s0) - lane);
+        j0 = s0 - lane;
+        if (CODES) db = dout + ((int64_t)(s0 / SPW) * 32 + lane) * (W > 0 ? W : 1);
+        if (puts) hb = static_cast<char*>(hcur) + (int64_t)j0 * SLOT;
+    }
+
+    // Step u of the chunk: the lane's column j = j0 + u (in range when FULLCHUNK).
     // dl holds the local costs of column j on entry and those of column j+1 on
     // exit: the next column's costs are computed between the links of this
     // column's min-plus chain, which is serial down the rows.
-    template <bool FULLCHUNK, bool MASK = false>
-    __device__ __forceinline__ void step(const u64* ring, int s, int src, int lane, int N, bool top,
-                                         void* hcur, uint32_t* dout)
+    template <bool FULLCHUNK, bool MASK = false, bool TRACK = false>
+    __device__ __forceinline__ void step(const u64* slot, int u, int lane, int N, bool top)
     {
         const float INF = inf_f();
         const float above = __shfl_up_sync(FULL, col[R - 1], 1);
-        const float tv = __shfl_sync(FULL, topv, src);
+        const float tv = __shfl_sync(FULL, topv, u);
         // above the matrix: +inf (DTW), 0 for Sub-DTW (a path may start in any column)
         const float top_in = MODE == kModeSubDirs ? 0.f : INF;
         const float up_in = lane == 0 ? (top ? top_in : tv) : above;
@@ -183,21 +228,18 @@ struct Band {
         int upc_in = 0, dgc_in = 0;
         if (MODE == kModePlen) {
             const int abovec = __shfl_up_sync(FULL, cnt[R - 1], 1);
-            const int tc = __shfl_sync(FULL, topc, src);
+            const int tc = __shfl_sync(FULL, topc, u);
             upc_in = lane == 0 ? tc : abovec;
             dgc_in = prev_upc;
             prev_upc = upc_in;
         }
-        const int j = s - lane;
+        const int j = j0 + u;
         u64 yy[D];
-        load_samples(ring, j + 1, yy);
-        uint32_t word[W > 0 ? W : 1];
-#pragma unroll
-        for (int w = 0; w < (W > 0 ? W : 1); ++w) word[w] = 0u;
+        load_samples(u + 1, yy);
+        uint32_t pl0 = 0u, pl1 = 0u;             // the step's code planes (in the low R bits)
         // partial chunks with a band read the band's columns (and the band)
         // from the warp's slot after the sample ring:
         // [jlo | jhi << 32, row0 | M << 32, bnd]
-        const u64* slot = ring + D * kRing;
         bool valid = true;
         int klo = 0, khi = R - 1;
         if (!FULLCHUNK && !BANDED) valid = j >= 0 && j < N;
@@ -224,8 +266,17 @@ struct Band {
                 float r = __fadd_rn(dl[k], m);
                 if (MASK && (k < klo || k > khi)) r = INF;     // outside the band
                 if (CODES) {
-                    word[k >> 5] |= ne_mask(dg, m) & (1u << (k & 31));
-                    word[(R + k) >> 5] |= ne_mask(up, m) & (1u << ((R + k) & 31));
+                    if (SIGNS) {
+                        // the sign of m - v (0 when equal, also at +inf: that NaN is positive)
+                        pl0 = __funnelshift_l(__float_as_uint(__fsub_rn(m, dg)), pl0, 1);
+                        pl1 = __funnelshift_l(__float_as_uint(__fsub_rn(m, up)), pl1, 1);
+                    } else if (R < 32) {
+                        pl0 |= ne_mask(dg, m) & (1u << (R - 1 - k));
+                        pl0 |= ne_mask(up, m) & (1u << ((2 * R - 1 - k) & 31));
+                    } else {
+                        pl0 |= ne_mask(dg, m) & (1u << (R - 1 - k));
+                        pl1 |= ne_mask(up, m) & (1u << (R - 1 - k));
+                    }
                 } else if (MODE == kModePlen) {
                     const int cl = cnt[k];
                     const int cn = 1 + (dg == m ? cdg : (up == m ? cup : cl));
@@ -238,35 +289,33 @@ struct Band {
                 col[k] = r;
                 if (k & 1) cost_pair(yy, k >> 1);      // rows k-1, k of column j+1
             }
-            if (MODE == kModeSubDirs && track) {
+            if (TRACK) {
                 const float v = pick_row<R>(col, kk);
-                if (v < best) { best = v; bestj = j; }
+                const bool less = v < best;
+                best = less ? v : best;
+                bestj = less ? j : bestj;
             }
-            if (lane == 31 && hcur != nullptr) {
+            if (puts) {
                 if (MODE == kModePlen)
-                    __stcg(reinterpret_cast<u64*>(hcur) + j, pack2(col[R - 1], __int_as_float(cnt[R - 1])));
+                    __stcg(reinterpret_cast<u64*>(hb) + u, pack2(col[R - 1], __int_as_float(cnt[R - 1])));
                 else
-                    __stcg(reinterpret_cast<float*>(hcur) + j, col[R - 1]);
+                    __stcg(reinterpret_cast<float*>(hb) + u, col[R - 1]);
             }
         } else {
 #pragma unroll
             for (int q = 0; q < Q; ++q) cost_pair(yy, q);
         }
         if (CODES) {
-            if (W == 0 && SPW == 2) {
-                if ((s & 1) == 0)
-                    half = word[0];
+            if (W < 2 && SIGNS) pl0 = R == 16 ? __byte_perm(pl0, pl1, 0x5410) : (pl1 << R) | pl0;
+            if (W == 0) {                    // (chunks start at multiples of 32)
+                if ((u & 1) == 0)
+                    half = pl0;
                 else
-                    __stcs(dout + (int64_t)(s >> 1) * 32 + lane, __byte_perm(half, word[0], 0x5410));
-            } else if (W == 0) {
-                const int sl = s & (SPW - 1);
-                half = sl == 0 ? word[0] : (half | (word[0] << (sl * 2 * R)));
-                if (sl == SPW - 1) __stcs(dout + (int64_t)(s / SPW) * 32 + lane, half);
+                    __stcs(db + (u >> 1) * 32, __byte_perm(half, pl0, 0x5410));
             } else if (W == 1) {
-                __stcs(dout + (int64_t)s * 32 + lane, word[0]);
+                __stcs(db + u * 32, pl0);
             } else {
-                __stcs(reinterpret_cast<uint2*>(dout) + (int64_t)s * 32 + lane,
-                       make_uint2(word[0], word[W > 1 ? 1 : 0]));
+                __stcs(reinterpret_cast<uint2*>(db) + u * 32, make_uint2(pl0, pl1));
             }
         }
     }
@@ -302,7 +351,6 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     st.topv = INF;
     st.topc = 0;
     st.half = 0u;
-    st.track = MODE == kModeSubDirs && last;
     st.kk = M - 1 - i0;
     st.best = INF;
     st.bestj = 0;
@@ -323,8 +371,8 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
         if (!top) { jtop_lo = lo_of(r0 - 1); jtop_hi = hi_of(r0 - 1); }
         if (i0 < M) { full_lo = lo_of(min(i0 + R - 1, M - 1)); full_hi = hi_of(i0); }
     }
+    u64* slot = ring + D * kRing;
     if (BANDED) {
-        u64* slot = ring + D * kRing;
         __syncwarp();
         if (lane == 0) {
             slot[0] = (u64)(uint32_t)jlo_b | ((u64)(uint32_t)jhi_b << 32);
@@ -340,14 +388,15 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     const int s_begin = max(0, (jlo_b - 1) & ~31);
     const int s_end = jhi_b + 32;           // one past the last step (column jhi_b in lane 31)
 
-    // hand-off rows: slot size 4 bytes (r), or 8 bytes ({r, cells}) with |pi|
-    constexpr int SLOT = MODE == kModePlen ? 8 : 4;
+    constexpr int SLOT = BandT::SLOT;
     char* hb = static_cast<char*>(p.hbuf);
     const char* hprev = top ? nullptr : hb + (pd.hbuf_off + (int64_t)(band - 1) * N) * SLOT;
     // a recomputed band reads its stored top row and produces no hand-off row
     void* hcur = (last || p.recompute || p.skip_handoff) ? nullptr : hb + (pd.hbuf_off + (int64_t)band * N) * SLOT;
     uint32_t* dout = BandT::CODES ? p.dirs + pd.dir_off + (int64_t)(band - p.band_lo) * band_dir_words(N, R)
                                          : nullptr;
+
+    st.puts = lane == 31 && hcur != nullptr;
 
     // Cycle samples go through the ring two chunks of 32 columns ahead of the
     // step that first reads them (a step also reads the next column), loaded
@@ -361,7 +410,13 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     };
     auto put_y = [&](int jj) {
 #pragma unroll
-        for (int c = 0; c < D; ++c) ring[c * kRing + (jj & (kRing - 1))] = pack2(ynext[c], ynext[c]);
+        for (int c = 0; c < D; ++c) {
+            u64* row = ring + c * kRing;
+            const u64 v = pack2(ynext[c], ynext[c]);
+            const int i = jj & 127;
+            row[i < 32 ? i + 128 : i] = v;
+            if (i < 36) row[i < 32 ? i : i + 128] = v;
+        }
     };
     auto load_t = [&](int jj) -> u64 {
         if (jj >= N) return 0;
@@ -376,10 +431,11 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     load_y(s_begin + lane + 64);
     if (!top) tnext = load_t(s_begin + lane);
     __syncwarp();
+    st.begin_chunk(ring, s_begin, lane, hcur, dout);
     {
         // local costs of the lane's first column (j = s_begin - lane)
         u64 yy[D];
-        st.load_samples(ring, s_begin - lane, yy);
+        st.load_samples(0, yy);
 #pragma unroll
         for (int q = 0; q < BandT::Q; ++q) st.cost_pair(yy, q);
     }
@@ -406,21 +462,26 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
                 tnext = load_t(jj + 32);
             }
         }
+        st.begin_chunk(ring, s0, lane, hcur, dout);
         // every lane in the band's columns and inside the band all chunk long
         const bool full = BANDED ? (s0 - 31 >= jlo_b && s0 + 31 <= jhi_b &&
                                     __all_sync(FULL, s0 - lane >= full_lo && s0 + 31 - lane <= full_hi))
                                  : (s0 >= 31 && s0 + 32 <= N);
-        if (full) {
-#pragma unroll 2
-            for (int u = 0; u < 32; ++u) st.template step<true>(ring, s0 + u, u, lane, N, top, hcur, dout);
-        } else {
-            const int n = min(32, s_end - s0);
-            if (BANDED) {
-                for (int u = 0; u < n; ++u) st.template step<false, true>(ring, s0 + u, u, lane, N, top, hcur, dout);
+        auto chunk = [&](auto track) {
+            constexpr bool TRACK = decltype(track)::value;
+            if (full) {
+#pragma unroll (R == 8 ? 4 : 2)
+                for (int u = 0; u < 32; ++u) st.template step<true, false, TRACK>(slot, u, lane, N, top);
             } else {
-                for (int u = 0; u < n; ++u) st.template step<false>(ring, s0 + u, u, lane, N, top, hcur, dout);
+                const int n = min(32, s_end - s0);
+#pragma unroll 1
+                for (int u = 0; u < n; ++u) st.template step<false, BANDED, TRACK>(slot, u, lane, N, top);
             }
-        }
+        };
+        if (MODE == kModeSubDirs && last)
+            chunk(std::true_type{});
+        else
+            chunk(std::false_type{});
     }
 
     constexpr int SPW = BandT::SPW;
@@ -441,18 +502,7 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
 #pragma unroll
             for (int k = 1; k < R; ++k)
                 if (k == kk) { v = st.col[k]; c = st.cnt[k]; }
-            if (p.cost_out) p.cost_out[pd.out] = v;
-            if (MODE == kModePlen) {
-                if (p.plen_out) p.plen_out[pd.out] = c;
-                if (p.score_out) p.score_out[pd.out] = __fdiv_rn(v, (float)c);
-            }
-            if (p.cost_matrix) {
-                int a = 0, rem = pd.out;
-                while (rem >= p.T - 1 - a) { rem -= p.T - 1 - a; ++a; }
-                const int bb = a + 1 + rem;
-                p.cost_matrix[(int64_t)a * p.T + bb] = v;
-                p.cost_matrix[(int64_t)bb * p.T + a] = v;
-            }
+            write_pair<MODE>(p, pd, v, c);
         }
     }
 }
@@ -461,11 +511,39 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
 // registers) where the prototype rows fit easily, two otherwise (the
 // software-pipelined step keeps enough independent work per warp).  R = 8
 // halves the prototype registers: four blocks (16 warps, <= 128 registers) up
-// to 6 channels.
+// to 4 channels, three up to 8 (at 6 the four spilled).
 template <int D, int R>
 constexpr int min_blocks()
 {
-    return R == 4 ? (D <= 8 ? 4 : 3) : R == 8 ? (D <= 6 ? 4 : (D <= 8 ? 3 : 2)) : ((R == 16 && D <= 4) ? 3 : 2);
+    return R == 8 ? (D <= 4 ? 4 : (D <= 8 ? 3 : 2)) : ((R == 16 && D <= 4) ? 3 : 2);
+}
+
+// The (place q in the work list's pair order, band) of an item.
+__device__ __forceinline__ void item_of(const DPParams& p, int item, int& q, int& band)
+{
+    if (p.group_pairs > 0) {
+        // groups of G pairs (in the work list's order), band-major within
+        // a group: a group's bands start in the order their producers
+        // do, and its items about fill the resident warps once (G = P:
+        // every pair's band b before any band b + 1, as under a band,
+        // where a pair has few bands ready at a time).  Every pair has the
+        // same bands here (one prototype); recompute runs the range
+        // [band_lo, band_lo + band_cnt) of each.  Band b - 1 of a pair is
+        // earlier in the list (no deadlock).
+        const int nb = p.recompute ? p.band_cnt : p.prefix[1] - p.prefix[0];
+        const int G = p.group_pairs;
+        const int g = item / (G * nb), q0 = g * G;
+        const int Gg = min(G, p.P - q0);
+        const int r = item - q0 * nb;
+        q = q0 + r % Gg;
+        band = (p.recompute ? p.band_lo : 0) + r / Gg;
+    } else if (p.recompute) {
+        q = item / p.band_cnt;
+        band = p.band_lo + item % p.band_cnt;
+    } else {
+        q = find_slot(p.prefix, p.P, item);
+        band = item - p.prefix[q];
+    }
 }
 
 template <int D, int R, int MODE, bool BANDED, int COST>
@@ -481,29 +559,7 @@ __global__ void __launch_bounds__(128, min_blocks<D, R>()) dtw_wavefront_kernel(
         if (item >= p.n_items) break;
         if (ld_volatile(&p.hdr->abort)) break;
         int q, band;
-        if (p.group_pairs > 0) {
-            // groups of G pairs (in the work list's order), band-major within
-            // a group: a group's bands start in the order their producers
-            // do, and its items about fill the resident warps once (G = P:
-            // every pair's band b before any band b + 1, as under a band,
-            // where a pair has few bands ready at a time).  Every pair has the
-            // same bands here (one prototype); recompute runs the range
-            // [band_lo, band_lo + band_cnt) of each.  Band b - 1 of a pair is
-            // earlier in the list (no deadlock).
-            const int nb = p.recompute ? p.band_cnt : p.prefix[1] - p.prefix[0];
-            const int G = p.group_pairs;
-            const int g = item / (G * nb), q0 = g * G;
-            const int Gg = min(G, p.P - q0);
-            const int r = item - q0 * nb;
-            q = q0 + r % Gg;
-            band = (p.recompute ? p.band_lo : 0) + r / Gg;
-        } else if (p.recompute) {
-            q = item / p.band_cnt;
-            band = p.band_lo + item % p.band_cnt;
-        } else {
-            q = find_slot(p.prefix, p.P, item);
-            band = item - p.prefix[q];
-        }
+        item_of(p, item, q, band);
         const PairDesc pd = p.pairs[p.order[q]];
         run_band<D, R, MODE, BANDED, COST>(p, pd, band, lane, ring);
     }
@@ -537,42 +593,31 @@ int occ_one(int block)
 template <int D, int R, bool BANDED, int COST>
 cudaError_t launch_mode(int mode, const DPParams& p, int grid, int block, cudaStream_t st)
 {
-    if constexpr (R == 4) {                  // Sub-DTW windows only (one pair: more, shorter bands)
-        if (mode == kModeSubDirs && !BANDED) return launch_one<D, 4, kModeSubDirs, false, COST>(p, grid, block, st);
-        return cudaErrorInvalidValue;
-    } else {
-        switch (mode) {
-            case kModeCost: return launch_one<D, R, kModeCost, BANDED, COST>(p, grid, block, st);
-            case kModePlen: return launch_one<D, R, kModePlen, BANDED, COST>(p, grid, block, st);
-            case kModeDirs: return launch_one<D, R, kModeDirs, BANDED, COST>(p, grid, block, st);
-            case kModeSubDirs:
-                if constexpr (!BANDED && (R == 16 || R == 8))
-                    return launch_one<D, R, kModeSubDirs, false, COST>(p, grid, block, st);
-                break;
-            default: break;
-        }
-        return cudaErrorInvalidValue;
+    switch (mode) {
+        case kModeCost: return launch_one<D, R, kModeCost, BANDED, COST>(p, grid, block, st);
+        case kModePlen: return launch_one<D, R, kModePlen, BANDED, COST>(p, grid, block, st);
+        case kModeDirs: return launch_one<D, R, kModeDirs, BANDED, COST>(p, grid, block, st);
+        case kModeSubDirs:
+            if constexpr (!BANDED && R <= 16) return launch_one<D, R, kModeSubDirs, false, COST>(p, grid, block, st);
+            break;
+        default: break;
     }
+    return cudaErrorInvalidValue;
 }
 
 template <int D, int R, bool BANDED, int COST>
 int occ_mode(int mode, int block)
 {
-    if constexpr (R == 4) {
-        if (mode == kModeSubDirs && !BANDED) return occ_one<D, 4, kModeSubDirs, false, COST>(block);
-        return 0;
-    } else {
-        switch (mode) {
-            case kModeCost: return occ_one<D, R, kModeCost, BANDED, COST>(block);
-            case kModePlen: return occ_one<D, R, kModePlen, BANDED, COST>(block);
-            case kModeDirs: return occ_one<D, R, kModeDirs, BANDED, COST>(block);
-            case kModeSubDirs:
-                if constexpr (!BANDED && (R == 16 || R == 8)) return occ_one<D, R, kModeSubDirs, false, COST>(block);
-                break;
-            default: break;
-        }
-        return 0;
+    switch (mode) {
+        case kModeCost: return occ_one<D, R, kModeCost, BANDED, COST>(block);
+        case kModePlen: return occ_one<D, R, kModePlen, BANDED, COST>(block);
+        case kModeDirs: return occ_one<D, R, kModeDirs, BANDED, COST>(block);
+        case kModeSubDirs:
+            if constexpr (!BANDED && R <= 16) return occ_one<D, R, kModeSubDirs, false, COST>(block);
+            break;
+        default: break;
     }
+    return 0;
 }
 
 // One set of instances: every padded channel count D (1, 2, 3 only for R = 32).
@@ -588,6 +633,7 @@ int occ_mode(int mode, int block)
             case 4: return FN<4, R, BANDED, COST>(__VA_ARGS__);               \
             case 6: return FN<6, R, BANDED, COST>(__VA_ARGS__);               \
             case 8: return FN<8, R, BANDED, COST>(__VA_ARGS__);               \
+            case 9: return FN<9, R, BANDED, COST>(__VA_ARGS__);               \
             case 12: return FN<12, R, BANDED, COST>(__VA_ARGS__);             \
             case 16: return FN<16, R, BANDED, COST>(__VA_ARGS__);             \
             default: break;                                                  \

@@ -73,15 +73,15 @@ __device__ __forceinline__ bool is_nan_bits(uint32_t bits) { return (bits & 0x7f
 // Spin (warp-uniform) until no lane reports `missing`; `reload` re-reads the
 // lane's slot and returns whether it is still missing.  Bounded: after `limit`
 // rounds, or once another warp raised the abort word, records a timeout and
-// returns false.
-template <typename Reload>
+// returns false.  The first FAST rounds poll without a pause.
+template <int FAST = 0, typename Reload>
 __device__ __forceinline__ bool wait_filled(bool missing, Reload reload, WsHeader* hdr, int where,
                                             long long limit = kSpinLimit)
 {
     if (!__any_sync(FULL, missing)) return true;
     long long spins = 0;
     for (;;) {
-        __nanosleep(64);
+        if (FAST == 0 || spins >= FAST) __nanosleep(64);
         if (missing) missing = reload();
         if (!__any_sync(FULL, missing)) return true;
         if (ld_volatile(&hdr->abort)) return false;
