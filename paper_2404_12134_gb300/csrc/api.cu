@@ -15,6 +15,7 @@
 #include "dba.cuh"
 #include "dtw_wavefront.cuh"
 #include "plan.cuh"
+#include "rows.cuh"
 #include "softdtw.cuh"
 
 namespace wts {
@@ -134,7 +135,9 @@ int check_opt(const wts_options* opt, int D)
 }
 
 // Layout of the workspace for one call (host side; mirrors the setup kernel).
-int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L)
+// fixed_rows: rows per lane 32 / 16 by the channel count where the options name
+// none, instead of the choice by the launch's size (rows.cuh).
+int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L, bool fixed_rows = false)
 {
     int rc = check_batch(Y, false);
     if (rc) return rc;
@@ -187,9 +190,20 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
         }
         L->cost_kind = WTS_COST_L2;
     }
+    const int64_t* o = Y->offsets_host;
+    // (checkpointed codes count their memory in bands, so they keep the rows)
+    if (!fixed_rows && (op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) &&
+        !(opt && (opt->rows_per_thread || opt->band > 0 || opt->dir_mode || opt->cost_kind != WTS_COST_SQEUCLID))) {
+        RowLoad load;
+        for (int a = 0; a < L->T; ++a) {
+            if (op != kOpPairwise) load.add(M, o[a + 1] - o[a]);
+            else
+                for (int b = a + 1; b < L->T; ++b) load.add(o[a + 1] - o[a], o[b + 1] - o[b]);
+        }
+        L->R = load.rows(D, op == kOpScore ? kRowPlen : (op == kOpPairwise ? kRowCost : kRowCodes), L->R);
+    }
     L->BR = 32 * L->R;
     L->M = M;
-    const int64_t* o = Y->offsets_host;
     // soft-DTW column checkpoints: the first store_pairs pairs of the work
     // list's order (longest first, or the batch order) keep R; the setup
     // kernel takes the same ranks
@@ -254,6 +268,9 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     L->rstore_floats = rs;
     // hand-off slot: r (4 bytes), or {r, path cells} (8 bytes) when |pi| is counted
     L->hbuf_bytes = (size_t)h * (op == kOpScore ? 8 : 4);
+    // four rows per lane: the same hand-off area for the score and the paths,
+    // so that one workspace of a small batch serves both
+    const size_t hbuf_room = op != kOpSubdtw && op != kOpSoft && L->R == 4 ? (size_t)h * 8 : L->hbuf_bytes;
     L->ebuf_bytes = op == kOpSoft ? (size_t)h * 16 : 0;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off = align256(off + bytes); return at; };
@@ -261,7 +278,7 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     L->off_pairs = take((size_t)L->P * sizeof(PairDesc));
     L->off_order = take((size_t)L->P * sizeof(int32_t));
     L->off_prefix = take((size_t)(L->P + 1) * sizeof(int32_t));
-    L->off_hbuf = take(L->hbuf_bytes);
+    L->off_hbuf = take(hbuf_room);
     if (op == kOpAlign || op == kOpDba || op == kOpSubdtw) {
         L->off_dirs = take((size_t)dw * sizeof(uint32_t));
         if (opt && opt->dir_mode == 1) {
@@ -296,6 +313,18 @@ int check_ws(const Layout& L, const void* ws, size_t bytes)
     if (((uintptr_t)ws & 255) != 0) return fail(WTS_EINVAL, "workspace must be 256-byte aligned");
     if (bytes < L.total) return fail(WTS_ENOMEM, "workspace has %zu bytes, needs %zu", bytes, L.total);
     return WTS_OK;
+}
+
+// The layout that a call runs with in the workspace it was given: a workspace
+// sized for another batch (a longer one's is reused for shorter ones) may hold
+// the fixed rows' layout only, and then those run.
+int call_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, size_t bytes, Layout* L)
+{
+    int rc = compute_layout(op, M, Y, opt, L);
+    if (rc || bytes >= L->total) return rc;
+    Layout F;
+    if (compute_layout(op, M, Y, opt, &F, true) == WTS_OK && bytes >= F.total) *L = F;
+    return ok();
 }
 
 struct DevInfo {
@@ -677,7 +706,7 @@ int anomaly_score(const float* B, int64_t M, const wts_batch* Y, const wts_optio
                   float* score, float* cost, int32_t* plen)
 {
     Layout L;
-    int rc = compute_layout(kOpScore, M, Y, opt, &L);
+    int rc = call_layout(kOpScore, M, Y, opt, workspace_bytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if (!B || !score) return fail(WTS_EINVAL, "B and score must not be NULL");
@@ -714,7 +743,7 @@ int dtw_align(const float* B, int64_t M, const wts_batch* Y, const wts_options* 
               float* cost, int32_t* plen, int32_t* jlo, int32_t* jhi)
 {
     Layout L;
-    int rc = compute_layout(kOpAlign, M, Y, opt, &L);
+    int rc = call_layout(kOpAlign, M, Y, opt, workspace_bytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if (!B || !jlo || !jhi) return fail(WTS_EINVAL, "B, jlo and jhi must not be NULL");
@@ -978,7 +1007,7 @@ int dba_iterate(const float* B_in, float* B_out, int64_t M, const wts_batch* Y, 
                 int32_t* counts, double* cost_before, float* cost)
 {
     Layout L;
-    int rc = compute_layout(kOpDba, M, Y, opt, &L);
+    int rc = call_layout(kOpDba, M, Y, opt, workspace_bytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if (!B_in || !B_out) return fail(WTS_EINVAL, "B_in and B_out must not be NULL");
@@ -1007,7 +1036,7 @@ int wts_pairwise_dtw(const wts_batch* Y, const wts_options* opt, void* workspace
                      void* stream, float* C)
 {
     Layout L;
-    int rc = compute_layout(kOpPairwise, 0, Y, opt, &L);
+    int rc = call_layout(kOpPairwise, 0, Y, opt, workspace_bytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if (!C) return fail(WTS_EINVAL, "C must not be NULL");
@@ -1455,7 +1484,7 @@ extern "C" int anomaly_score_noalloc(const float* B, int64_t M, const wts_batch*
     o.score_via_codes = 0;
     opt = &o;
     Layout L;
-    int rc = compute_layout(kOpScore, M, Y, opt, &L);
+    int rc = call_layout(kOpScore, M, Y, opt, kNoAllocScratchBytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if (!B || !score) return fail(WTS_EINVAL, "B and score must not be NULL");

@@ -108,7 +108,7 @@ constexpr int kSlot = 4;     // u64 words after a warp's ring: its band's column
 
 
 
-constexpr int kSignD = 3;
+constexpr int kSignD = 4;
 
 // c[k] for a k known only at run time, by a binary tree of selects on the bits
 // of k (R - 1 selects, no local memory)
