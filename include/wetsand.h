@@ -204,7 +204,7 @@ int anomaly_score(const float* B, int64_t M, const wts_batch* Y, const wts_optio
  *   jlo  [T][M], jhi [T][M]      out (int32); with every code stored
  *                                (dir_mode 0) the walk reads the jhi values
  *                                found there on entry as guesses of where
- *                                the path enters rows 2048 apart (a repeated
+ *                                the path enters rows 256 to 2048 apart (a repeated
  *                                call on the same arrays walks faster); any
  *                                contents are safe and the result does not
  *                                depend on them

@@ -283,9 +283,12 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
         L->off_dirs = take((size_t)dw * sizeof(uint32_t));
         if (opt && opt->dir_mode == 1) {
             L->group_bands = opt->ckpt_bands ? opt->ckpt_bands : 16;
-            L->off_btstate = take((size_t)L->T * 3 * sizeof(int32_t));
+            L->off_btstate = take((size_t)L->T * sizeof(int32_t));
+            L->nseg = (int)cdiv(std::min<int64_t>(M, (int64_t)L->group_bands * L->BR),
+                                bt_seg_rows((int64_t)L->group_bands * L->BR));
+            L->off_seg = take((size_t)L->P * L->nseg * 4 * sizeof(int32_t));
         } else if (op != kOpSubdtw) {
-            L->nseg = (int)cdiv(M, kBtSegRows);
+            L->nseg = (int)cdiv(M, bt_seg_rows(M));
             L->off_seg = take((size_t)L->P * L->nseg * 4 * sizeof(int32_t));
         }
     }
@@ -459,6 +462,20 @@ int launch_dp(int mode, const Layout& L, const DPParams& p0, const wts_options* 
     return WTS_OK;
 }
 
+// The rounds of a segmented walk and its last kernel.
+cudaError_t segmented_walk(BTParams bt, cudaStream_t st)
+{
+    Prof pr("backtrack", st);
+    pr.kernels = bt.nseg + 1;
+    for (int r = 0; r < bt.nseg; ++r) {
+        bt.round = r;
+        const cudaError_t e = launch_backtrack(bt, st);
+        if (e != cudaSuccess) return e;
+    }
+    bt.round = bt.nseg - 1;
+    return launch_backtrack_seg_final(bt, st);
+}
+
 // Shared body of dtw_align and dba_iterate: directions + backtrack.
 int align_into(const Layout& L, char* ws, const float* B, const wts_batch* Y, const wts_options* opt,
                cudaStream_t st, float* cost, int32_t* plen, int32_t* jlo, int32_t* jhi)
@@ -488,20 +505,14 @@ int align_into(const Layout& L, char* ws, const float* B, const wts_batch* Y, co
         // whose start changed), then |pi| from the ranges; a single segment
         // is one plain walk per pair
         bt.nseg = L.nseg > 1 ? L.nseg : 0;
-        bt.seg_rows = kBtSegRows;
+        bt.seg_rows = bt_seg_rows(L.M);
         bt.seg = reinterpret_cast<int32_t*>(ws + L.off_seg);
+        bt.first = 1;
         if (bt.nseg == 0) {
             Prof pr("backtrack", st);
             e = launch_backtrack(bt, st);
         } else {
-            Prof pr("backtrack", st);
-            pr.kernels = L.nseg + 1;
-            for (int r = 0; r < L.nseg; ++r) {
-                bt.round = r;
-                e = launch_backtrack(bt, st);
-                if (e != cudaSuccess) break;
-            }
-            if (e == cudaSuccess) e = launch_backtrack_seg_final(bt, st);
+            e = segmented_walk(bt, st);
         }
         if (e != cudaSuccess) return cuda_fail(e, "backtrack launch");
         return WTS_OK;
@@ -515,6 +526,9 @@ int align_into(const Layout& L, char* ws, const float* B, const wts_batch* Y, co
     const int nb = (int)cdiv(L.M, L.BR);
     const int G = L.group_bands;
     bt.state = reinterpret_cast<int32_t*>(ws + L.off_btstate);
+    bt.seg = reinterpret_cast<int32_t*>(ws + L.off_seg);
+    bt.nseg = L.nseg;
+    bt.seg_rows = bt_seg_rows((int64_t)G * L.BR);
     for (int hi = nb; hi > 0; hi -= G) {
         const int lo = hi - G > 0 ? hi - G : 0;
         DPParams r = p;
@@ -531,10 +545,7 @@ int align_into(const Layout& L, char* ws, const float* B, const wts_batch* Y, co
         bt.band_lo = lo;
         bt.band_hi = hi;
         bt.first = hi == nb;
-        {
-            Prof pr("backtrack", st);
-            e = launch_backtrack(bt, st);
-        }
+        e = segmented_walk(bt, st);
         if (e != cudaSuccess) return cuda_fail(e, "backtrack launch");
     }
     return WTS_OK;

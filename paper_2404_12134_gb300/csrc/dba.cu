@@ -37,8 +37,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase)
 // band, so a window of kBtWords / 32 consecutive word rows (one contiguous
 // block of global memory) is brought into shared memory by one bulk
 // asynchronous copy (completion on an mbarrier, bounded wait) and the walk
-// reads it; every lane walks the same path, and the lanes look ahead along a
-// run of equal moves (one vote per run).
+// reads it; every lane walks the same path, and the lanes look ahead along
+// runs of equal moves (one vote per run).
 // Row i's range is [jlo(i), jhi(i)]: jhi when the walk enters the row, jlo
 // when it leaves it (Definition "Alignment path": monotone, so each row's
 // columns are contiguous).
@@ -63,33 +63,40 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
+    // the lane's look-ahead: u moves of its group's kind (0 diagonal, 1 up, 2 left)
+    const int group = lane < 16 ? 0 : (lane < 24 ? 1 : 2);
+    const int u = lane - (group == 0 ? 0 : (group == 1 ? 16 : 24));
+    const bool g_i = group != 2, g_j = group != 1;
+    const int u_i = g_i ? u : 0, u_j = g_j ? u : 0;
     uint32_t phase = 0;
     bool failed = false;
     const int units = p.nseg > 0 ? p.P * p.nseg : p.P;
-    for (int u = blockIdx.x * kBtWarps + wid; u < units && !failed; u += gridDim.x * kBtWarps) {
-        const int q = p.nseg > 0 ? u / p.nseg : u;
+    for (int un = blockIdx.x * kBtWarps + wid; un < units && !failed; un += gridDim.x * kBtWarps) {
+        const int q = p.nseg > 0 ? un / p.nseg : un;
         const PairDesc pd = p.pairs[q];
         const int N = pd.N;
         int32_t* jlo = p.jlo + (int64_t)pd.out * p.M;
         int32_t* jhi = p.jhi + (int64_t)pd.out * p.M;
         int i, j, len;
-        int i_lo = p.band_lo * 32 * R;
-        int32_t* sg = p.nseg > 0 ? p.seg + 4 * (int64_t)u : nullptr;
+        const int row_lo = p.band_lo * 32 * R, row_hi = min((int64_t)pd.M, (int64_t)p.band_hi * 32 * R);
+        int i_lo = row_lo;
+        int32_t* sg = p.nseg > 0 ? p.seg + 4 * (int64_t)un : nullptr;
         const int cur = p.round & 1;
         bool mergeable = false, merged = false;
         int prev_exit = -1;
         if (p.nseg > 0) {
-            // segment sk: rows [sk * seg_rows, top]; the last one holds (M-1, N-1)
-            const int sk = u - q * p.nseg;
-            const int top = min(pd.M, (sk + 1) * p.seg_rows) - 1;
-            i_lo = sk * p.seg_rows;
+            // segment sk: rows [row_lo + sk * seg_rows, top]; the last one holds the group's last row
+            const int sk = un - q * p.nseg;
+            i_lo = row_lo + sk * p.seg_rows;
+            if (i_lo >= row_hi) continue;
+            const int top = min(row_hi, i_lo + p.seg_rows) - 1;
             int start;
-            if (top == pd.M - 1) {
-                if (p.round > 0) {                   // walked from the path's end in round 0
+            if (top == row_hi - 1) {
+                if (p.round > 0) {                   // walked from the path's entry in round 0
                     if (lane == 0) sg[1 + cur] = sg[2 - cur];
                     continue;
                 }
-                start = N - 1;
+                start = p.first ? N - 1 : p.state[q];
             } else if (p.round == 0) {
                 // a guess: the column this row was entered at by the previous
                 // walk of this pair (the ranges of an earlier call on the same
@@ -97,7 +104,7 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
                 start = jhi[top];
                 if (start < 0 || start >= N) start = (int)((int64_t)top * (N - 1) / max(pd.M - 1, 1));
             } else {
-                start = p.seg[4 * (int64_t)(u + 1) + 2 - cur];     // exit of the segment above, last round
+                start = p.seg[4 * (int64_t)(un + 1) + 2 - cur];     // exit of the segment above, last round
                 if (start == sg[0]) {                // unchanged: the walk recorded stands
                     if (lane == 0) sg[1 + cur] = sg[2 - cur];
                     continue;
@@ -120,7 +127,7 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
             }
             i = top; j = start; len = 0;
             if (lane == 0) { jhi[i] = j; sg[0] = start; }
-        } else if (p.state == nullptr || p.first) {
+        } else {
             i = pd.M - 1; j = p.subseq ? p.bstar[pd.out] : N - 1; len = 0;
             if (j < 0 || j >= N) {                    // b* is not a column of this cycle: no walk
                 if (lane == 0) {
@@ -130,9 +137,6 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
                 continue;
             }
             if (lane == 0) jhi[i] = j;
-        } else {
-            i = p.state[3 * q]; j = p.state[3 * q + 1]; len = p.state[3 * q + 2];
-            if (i < 0 || len < 0) continue;          // finished, or failed earlier
         }
         int band = -1, wlo = 0, whi = -1;           // word rows in the window
         bool left_group = false;
@@ -167,69 +171,97 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
                     break;
                 }
             }
-            // cell (ii, jj) of the window: lane t = (ii mod BR) / R, row k =
-            // ii mod R, step s = jj + t
-            auto code_at = [&](int ii, int jj, uint32_t& nd, uint32_t& nu) {
-                const int tt = (ii >> LOG_R) & 31;
-                const int kk = ii & (R - 1);
-                const int ss = jj + tt;
-                const uint32_t* wp = win + ((ss / SPW - wlo) * 32 + tt) * W;
-                if (R == 4) {
-                    const uint32_t w1 = wp[0] << ((ss % SPW) * 2 * R + 2 * kk);
-                    nd = w1 >> 31;
-                    nu = (w1 >> 30) & 1u;
-                    return;
-                }
+            // away from the window's and the rows' ends: the same runs without a check
+            // (in a loop of its own: a warp walking alone is bound by the chain of
+            // dependent instructions, about 5 cycles each)
+            const int fi = max(b << (LOG_R + 5), i_lo + 1) + 16;
+            if (!mergeable && i >= fi && j >= 17 && j + ((i >> LOG_R) & 31) >= wlo * SPW + 21) {
+                const uint32_t* win0 = win - wlo * 32 * W;
+                int taken = 0;
+                do {
+                    const int iu = i - u_i, ju = j - u_j;
+                    const int tt = (iu >> LOG_R) & 31;
+                    const int ss = ju + tt;
+                    const uint32_t* wp = win0 + ((ss / SPW) * 32 + tt) * W;
+                    const int kk = iu & (R - 1);
+                    // "not diag" and "not up" of the cell at fixed places of x
+                    uint32_t x;
+                    if (R == 32) x = ((wp[0] << kk) & 0x80000000u) | (((wp[W - 1] << kk) >> 1) & 0x40000000u);
+                    else x = wp[0] << (R == 4 ? (ss % SPW) * 2 * R + 2 * kk : R == 8 ? kk + 16 - (ss & 1) * 16 : kk);
+                    constexpr uint32_t ND = R == 16 ? 0x8000u : (R == 8 ? 0x800000u : 0x80000000u);
+                    constexpr uint32_t NU = R == 16 || R == 8 ? 0x80000000u : 0x40000000u;
+                    const uint32_t mask = group == 0 ? ND : (ND | NU);
+                    const uint32_t want = group == 0 ? 0u : (group == 1 ? ND : (ND | NU));
+                    const uint32_t votes = __ballot_sync(FULL, (x & mask) == want);
+                    const int base = __ffs(votes & 0x01010001u) - 1;
+                    const int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
+                    const int di = base != 24, dj = base != 16;
+                    if (di && lane >= base && lane < base + run) {
+                        jlo[iu] = ju;
+                        jhi[iu - 1] = ju - dj;
+                    }
+                    i -= di ? run : 0;
+                    j -= dj ? run : 0;
+                    taken += run;
+                } while (i >= fi && j >= 17 && j + ((i >> LOG_R) & 31) >= wlo * SPW + 21);
+                len += taken - 1;
+                continue;
+            }
+            // Runs: the lanes read ahead along all three kinds of move at once,
+            // 16 cells on the diagonal, 8 up, 8 left (lane u of a group the cell
+            // that u moves of its kind would reach); a lane agrees if its cell is
+            // in the window and codes the group's move and, past the first, the
+            // move is an ordinary one (not out of the grid, not out of the rows
+            // loaded).  The first lane of one group agrees, which is the cell's
+            // own move, and the lanes that agree after it are the run: the same
+            // walk as one cell at a time, with one shared-memory read and one
+            // vote per run (the read of the cell, then of its run, took two).
+            const int iu = i - u_i, ju = j - u_j;
+            const int tt = (iu >> LOG_R) & 31;
+            const int ss = ju + tt;
+            const bool here = iu >= (b << (LOG_R + 5)) && ju >= 0 && ss >= wlo * SPW;
+            // cell (iu, ju) of the window: lane t = (iu mod BR) / R, row k = iu
+            // mod R, step s = ju + t
+            const uint32_t* wp = win + (here ? ((ss / SPW - wlo) * 32 + tt) * W : 0);
+            const int kk = iu & (R - 1);
+            uint32_t nd, nu;
+            if (R == 4) {
+                const uint32_t w1 = wp[0] << ((ss % SPW) * 2 * R + 2 * kk);
+                nd = w1 >> 31;
+                nu = (w1 >> 30) & 1u;
+            } else {
                 const uint32_t w0 = R < 16 ? wp[0] >> ((ss % SPW) * 2 * R) : wp[0];
                 nd = (w0 >> (R - 1 - kk)) & 1u;
                 nu = R <= 16 ? (w0 >> (2 * R - 1 - kk)) & 1u : (wp[W - 1] >> (R - 1 - kk)) & 1u;
-            };
-            uint32_t nd, nu;
-            code_at(i, j, nd, nu);
+            }
             // codes: diag (nd = 0) moves up-left, up (nd = 1, nu = 0) moves up,
             // left (nd = nu = 1) moves left
-            const int di = (nd == 0u || nu == 0u) ? 1 : 0;
-            const int dj = (nd == 0u || nu == 1u) ? 1 : 0;
+            const int kind = nd == 0u ? 0 : (nu == 0u ? 1 : 2);
+            const bool agree = here && kind == group &&
+                               (u == 0 || ((!g_i || (iu > 0 && iu - 1 >= i_lo)) && (!g_j || ju > 0)));
+            const uint32_t votes = __ballot_sync(FULL, agree);
+            const int base = __ffs(votes & 0x01010001u) - 1;       // the group's first lane
+            const int di = base != 24, dj = base != 16;
             // Sub-DTW: a move up from row 0 reaches the free start
             if (p.subseq && i == 0 && di) break;
             // a valid code matrix only moves left on row 0 and only up on
             // column 0; anything else is reported as |pi| = -1
             if ((i == 0 && di) || (j == 0 && dj)) { len = -1; break; }
-            // Runs: lane u > 0 reads the cell c_u = (i - u di, j - u dj) that u
-            // more moves of the same kind would reach, and agrees if that cell
-            // is in the window, codes the same move, and the move from it is an
-            // ordinary one (not the path's start, not out of the grid, not out
-            // of the rows loaded).  The moves of c_0 .. c_{run-1} are then
-            // taken at once, run = the first lane that does not agree: the same
-            // walk as one cell at a time, with one shared-memory round trip and
-            // one vote per run; lane u writes the rows that c_u leaves.
-            const int iu = i - lane * di, ju = j - lane * dj;
-            bool agree = false;
-            if (lane > 0 && iu >= 0 && ju >= 0 && (iu | ju) != 0 && (iu >> (LOG_R + 5)) == band) {
-                const int ru = (ju + ((iu >> LOG_R) & 31)) / SPW;
-                if (ru >= wlo && ru <= whi) {
-                    uint32_t ndu, nuu;
-                    code_at(iu, ju, ndu, nuu);
-                    const int diu = (ndu == 0u || nuu == 0u) ? 1 : 0;
-                    const int dju = (ndu == 0u || nuu == 1u) ? 1 : 0;
-                    agree = diu == di && dju == dj && !(iu == 0 && di) && !(ju == 0 && dj) && iu - di >= i_lo;
-                }
-            }
-            const uint32_t votes = __ballot_sync(FULL, agree) | 1u;
-            int run = votes == FULL ? 32 : __ffs(~votes) - 1;
+            int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
             // a re-walk: does the move of c_u enter a row at a cell of the
             // previous walk (read before this run's writes)?
+            const bool mine = lane >= base && lane < base + run && di;
             uint32_t mv = 0u;
             if (mergeable) {                         // warp-uniform
                 bool mg = false;
-                if (di && lane < run && iu - 1 >= i_lo) {
+                if (mine && iu - 1 >= i_lo) {
                     const int je = ju - dj;
                     mg = jlo[iu - 1] <= je && je <= jhi[iu - 1];
                 }
                 mv = __ballot_sync(FULL, mg);
-                if (mv) run = __ffs(mv);             // up to and including the first such move
+                if (mv) run = __ffs(mv) - base;      // up to and including the first such move
             }
-            if (di && lane < run) {
+            if (mine && lane < base + run) {
                 jlo[iu] = ju;
                 jhi[iu - 1] = ju - dj;
             }
@@ -251,10 +283,6 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
             }
             continue;
         }
-        if (left_group) {
-            if (lane == 0) { p.state[3 * q] = i; p.state[3 * q + 1] = j; p.state[3 * q + 2] = len; }
-            continue;
-        }
         if (lane == 0) {
             if (p.subseq) {
                 if (len > 0) jlo[0] = j;
@@ -263,7 +291,6 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
                 jlo[0] = 0;
             }
             if (p.plen) p.plen[pd.out] = len;
-            if (p.state) { p.state[3 * q] = -1; p.state[3 * q + 2] = len; }
         }
     }
 }
@@ -280,7 +307,8 @@ __global__ void __launch_bounds__(128) bt_seg_final_kernel(BTParams p)
     if (p.hdr != nullptr && ld_volatile(&p.hdr->abort)) return;      // nothing was walked
     const PairDesc pd = p.pairs[q];
     const int last = (p.round & 1);                  // exit slot of the last round
-    const int nseg = (int)((pd.M + p.seg_rows - 1) / p.seg_rows);
+    const int rows = min((int64_t)pd.M, (int64_t)p.band_hi * 32 * p.R) - p.band_lo * 32 * p.R;
+    const int nseg = (rows + p.seg_rows - 1) / p.seg_rows;
     bool bad = false;
     for (int k = lane; k < nseg; k += 32) {
         const int32_t* sg = p.seg + 4 * ((int64_t)q * p.nseg + k);
@@ -288,6 +316,8 @@ __global__ void __launch_bounds__(128) bt_seg_final_kernel(BTParams p)
         if (k + 1 < nseg && sg[0] != p.seg[4 * ((int64_t)q * p.nseg + k + 1) + 1 + last]) bad = true;
     }
     bad = __any_sync(FULL, bad);
+    if (p.state != nullptr && lane == 0) p.state[q] = bad ? -1 : p.seg[4 * (int64_t)q * p.nseg + 1 + last];
+    if (p.band_lo > 0) return;                       // rows below are still to be walked
     const int32_t* jlo = p.jlo + (int64_t)pd.out * p.M;
     const int32_t* jhi = p.jhi + (int64_t)pd.out * p.M;
     long long cells = 0;
