@@ -244,6 +244,7 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
         }
         const int64_t nb = cdiv(Mp, L->BR);
         items += nb;
+        L->max_bands = std::max(L->max_bands, (int)nb);
         h += pair_hbuf_slots(nb, Np);
         if (op == kOpAlign || op == kOpDba || op == kOpSubdtw) {
             const int64_t G = (opt && opt->dir_mode == 1) ? (opt->ckpt_bands ? opt->ckpt_bands : 16) : 0;
@@ -443,15 +444,17 @@ int launch_dp(int mode, const Layout& L, const DPParams& p0, const wts_options* 
     int rc = grid_for(mode, L, opt, &grid, &block, p0.n_items);
     if (rc) return rc;
     DPParams p = p0;
-    // Every pair of a shared-prototype launch has the same bands: take the
-    // pairs in groups whose items about fill the resident warps once,
+    // Take the pairs in groups whose items about fill the resident warps once,
     // band-major within a group (measured: batched DBA, 200 x 25k x 6 ch,
-    // wavefront 74.1 -> 70.7 ms against pair after pair).  Under a band
-    // every pair's band b comes before any band b + 1 (one group).
-    if (L.op != kOpPairwise && L.M > 0) {
-        const int64_t nb = p.recompute ? p.band_cnt : cdiv(L.M, L.BR);
+    // wavefront 74.1 -> 70.7 ms against pair after pair; the pairwise matrix of
+    // 16 such cycles 43.5 -> 41.8 ms).  Under a band every pair's band b comes before
+    // any band b + 1 (one group).
+    const int64_t nb = p.recompute ? p.band_cnt : L.max_bands;
+    if ((int64_t)L.P * nb < ((int64_t)1 << 31)) {
         const int64_t warps = (int64_t)grid * (block / 32);
         p.group_pairs = p.banded ? L.P : (int)std::max<int64_t>(1, std::min<int64_t>(L.P, warps / nb));
+        p.group_bands = (int)nb;
+        if (!p.recompute) p.n_items = (int)(L.P * nb);
     }
     cudaError_t e;
     {

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(128, D <= 8 ? 3 : 2) dtw_lean_kernel(DPParams 
         int q, band;
         item_of(p, item, q, band);
         const PairDesc pd = p.pairs[p.order[q]];
-        lean_band<D, R, MODE, COST>(p, pd, band, lane, ring);
+        if (band < pd.nbands) lean_band<D, R, MODE, COST>(p, pd, band, lane, ring);
     }
 }
 

@@ -526,11 +526,12 @@ __device__ __forceinline__ void item_of(const DPParams& p, int item, int& q, int
         // a group: a group's bands start in the order their producers
         // do, and its items about fill the resident warps once (G = P:
         // every pair's band b before any band b + 1, as under a band,
-        // where a pair has few bands ready at a time).  Every pair has the
-        // same bands here (one prototype); recompute runs the range
-        // [band_lo, band_lo + band_cnt) of each.  Band b - 1 of a pair is
-        // earlier in the list (no deadlock).
-        const int nb = p.recompute ? p.band_cnt : p.prefix[1] - p.prefix[0];
+        // where a pair has few bands ready at a time).  A pair of fewer than
+        // group_bands bands (pairwise: the rows are a cycle) leaves its last
+        // items empty; recompute runs the range [band_lo, band_lo + band_cnt)
+        // of each pair.  Band b - 1 of a pair is earlier in the list (no
+        // deadlock).
+        const int nb = p.recompute ? p.band_cnt : p.group_bands;
         const int G = p.group_pairs;
         const int g = item / (G * nb), q0 = g * G;
         const int Gg = min(G, p.P - q0);
@@ -561,7 +562,7 @@ __global__ void __launch_bounds__(128, min_blocks<D, R>()) dtw_wavefront_kernel(
         int q, band;
         item_of(p, item, q, band);
         const PairDesc pd = p.pairs[p.order[q]];
-        run_band<D, R, MODE, BANDED, COST>(p, pd, band, lane, ring);
+        if (band < pd.nbands) run_band<D, R, MODE, BANDED, COST>(p, pd, band, lane, ring);
     }
 }
 

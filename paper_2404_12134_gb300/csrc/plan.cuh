@@ -53,6 +53,7 @@ struct Layout {
     int d = 0, D = 0, R = 0, BR = 0;
     int64_t M = 0;        // prototype length (shared-prototype ops)
     int64_t n_items = 0;  // total (pair, band) items
+    int max_bands = 0;    // the most bands of a pair
     int64_t hbuf_slots = 0, dir_words = 0, rstore_floats = 0;
     size_t hbuf_bytes = 0, ebuf_bytes = 0;
     size_t off_hdr = 0, off_pairs = 0, off_order = 0, off_prefix = 0;
