@@ -82,8 +82,8 @@ typedef struct wts_options {
     int32_t rows_per_thread;       /* prototype rows held per lane: 8, 16 or 32 (32 needs d <= 3); 4 for Sub-DTW only;
                                       0 = the library's choice: for anomaly_score, dtw_align, dba_iterate and the
                                       pairwise matrix by the launch's size (4, 8, 16 or 32; few rows while the warps
-                                      are few), 32 if d <= 2 and else 16 with dir_mode = 1, 16 with a band or the
-                                      l2 norm.  Results do not depend on it.  A workspace too small for that choice
+                                      are few), 32 if d <= 2 and else 16 with dir_mode = 1, 16 with a band; with the
+                                      l2 norm 4, 16 for the score, Sub-DTW, a band and dir_mode = 1.  Results do not depend on it.  A workspace too small for that choice
                                       but large enough for 32 / 16 rows is accepted and runs those.  Soft-DTW does
                                       not use it: 8 rows per lane, 4 under a band narrower than 0.45 */
     int32_t warps_per_block;       /* 0 = 4; 1..4 */
@@ -112,8 +112,8 @@ typedef struct wts_options {
     int32_t cost_kind;             /* local cost delta(b_i, y_j) (Definition "Distance Matrix", Sec. 3.2):
                                       WTS_COST_SQEUCLID (0, default) = sum_c (b_ic - y_jc)^2;
                                       WTS_COST_L2 (1) = its IEEE square root, the l2 norm.  Every DTW,
-                                      Sub-DTW and soft-DTW operation; the DTW kernels then hold 16 rows per
-                                      lane (rows_per_thread 0 or 16, else WTS_EINVAL).  The soft-DTW
+                                      Sub-DTW and soft-DTW operation; the DTW operations then take
+                                      rows_per_thread 0 or 16 (else WTS_EINVAL).  The soft-DTW
                                       gradient of the norm is (b_ic - y_jc) / delta, taken as 0 where
                                       delta = 0.  dba_iterate still averages the aligned samples (the mean
                                       minimises the squared cost only, so the DBA cost need not decrease). */

@@ -193,14 +193,22 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     const int64_t* o = Y->offsets_host;
     // (checkpointed codes count their memory in bands, so they keep the rows)
     if (!fixed_rows && (op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) &&
-        !(opt && (opt->rows_per_thread || opt->band > 0 || opt->dir_mode || opt->cost_kind != WTS_COST_SQEUCLID))) {
-        RowLoad load;
-        for (int a = 0; a < L->T; ++a) {
-            if (op != kOpPairwise) load.add(M, o[a + 1] - o[a]);
-            else
-                for (int b = a + 1; b < L->T; ++b) load.add(o[a + 1] - o[a], o[b + 1] - o[b]);
+        !(opt && (opt->rows_per_thread || opt->band > 0 || opt->dir_mode)) && !(op == kOpScore && L->cost_kind)) {
+        if (L->cost_kind == WTS_COST_L2) {
+            // four rows at every size: the square roots outweigh a step's fixed
+            // work, and sixteen rows of them spill (ns of a step at full issue, 4
+            // against 16 rows: d = 1 66 / 288, d = 6 98 / 468, d = 16 188 / 2136;
+            // 24 cycles of 8.2k x 6 ch: 3.9 against 8.0 ms)
+            L->R = 4;
+        } else {
+            RowLoad load;
+            for (int a = 0; a < L->T; ++a) {
+                if (op != kOpPairwise) load.add(M, o[a + 1] - o[a]);
+                else
+                    for (int b = a + 1; b < L->T; ++b) load.add(o[a + 1] - o[a], o[b + 1] - o[b]);
+            }
+            L->R = load.rows(D, op == kOpScore ? kRowPlen : (op == kOpPairwise ? kRowCost : kRowCodes), L->R);
         }
-        L->R = load.rows(D, op == kOpScore ? kRowPlen : (op == kOpPairwise ? kRowCost : kRowCodes), L->R);
     }
     L->BR = 32 * L->R;
     L->M = M;
@@ -271,7 +279,8 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     L->hbuf_bytes = (size_t)h * (op == kOpScore ? 8 : 4);
     // four rows per lane: the same hand-off area for the score and the paths,
     // so that one workspace of a small batch serves both
-    const size_t hbuf_room = op != kOpSubdtw && op != kOpSoft && L->R == 4 ? (size_t)h * 8 : L->hbuf_bytes;
+    const size_t hbuf_room = op != kOpSubdtw && op != kOpSoft && L->R == 4 && !L->cost_kind ? (size_t)h * 8
+                                                                                            : L->hbuf_bytes;
     L->ebuf_bytes = op == kOpSoft ? (size_t)h * 16 : 0;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off = align256(off + bytes); return at; };

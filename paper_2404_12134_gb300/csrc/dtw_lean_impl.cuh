@@ -339,13 +339,13 @@ int lean_occ_one(int block)
     return n;
 }
 
-#define WTS_LEAN_SWITCH(FN, ...)                                                   \
-    switch (mode) {                                                                \
-        case kModeCost: return FN<D, R, kModeCost, COST>(__VA_ARGS__);              \
-        case kModePlen: return FN<D, R, kModePlen, COST>(__VA_ARGS__);              \
-        case kModeDirs: return FN<D, R, kModeDirs, COST>(__VA_ARGS__);              \
-        case kModeSubDirs: return FN<D, R, kModeSubDirs, COST>(__VA_ARGS__);        \
-        default: break;                                                            \
+// (the l2 norm: codes and cost only)
+#define WTS_LEAN_SWITCH(FN, ...)                                                       \
+    if (mode == kModeCost) return FN<D, R, kModeCost, COST>(__VA_ARGS__);               \
+    if (mode == kModeDirs) return FN<D, R, kModeDirs, COST>(__VA_ARGS__);               \
+    if constexpr (COST != kCostL2) {                                                   \
+        if (mode == kModePlen) return FN<D, R, kModePlen, COST>(__VA_ARGS__);           \
+        if (mode == kModeSubDirs) return FN<D, R, kModeSubDirs, COST>(__VA_ARGS__);     \
     }
 
 template <int D, int R, int COST>

@@ -8,6 +8,7 @@ namespace wts {
 cudaError_t launch_dtw_wavefront(int mode, int D, int R, const DPParams& p, int grid, int block, cudaStream_t st)
 {
     if (p.cost_kind == kCostL2) {
+        if (R == 4 && !p.banded) return wf_launch_l2r4(mode, D, p, grid, block, st);
         if (R != 16) return cudaErrorInvalidValue;
         return p.banded ? wf_launch_l2b(mode, D, p, grid, block, st) : wf_launch_l2(mode, D, p, grid, block, st);
     }
@@ -25,6 +26,7 @@ cudaError_t launch_dtw_wavefront(int mode, int D, int R, const DPParams& p, int 
 int dtw_wavefront_max_blocks_per_sm(int mode, int D, int R, int block, int banded, int cost_kind)
 {
     if (cost_kind == kCostL2) {
+        if (R == 4 && !banded) return wf_occ_l2r4(mode, D, block);
         if (R != 16) return 0;
         return banded ? wf_occ_l2b(mode, D, block) : wf_occ_l2(mode, D, block);
     }

@@ -60,6 +60,7 @@ int dtw_wavefront_max_blocks_per_sm(int mode, int D, int R, int block, int bande
     X(r16b)   /* R = 16, band,    squared l2 */ \
     X(r32)    /* R = 32, no band, squared l2 (d <= 3) */ \
     X(l2)     /* R = 16, no band, l2 norm */ \
+    X(l2r4)   /* R = 4,  no band, l2 norm (codes and cost only) */ \
     X(l2b)    /* R = 16, band,    l2 norm */
 #define WTS_WF_DECL(TAG)                                                                                  \
     cudaError_t wf_launch_##TAG(int mode, int D, const DPParams& p, int grid, int block, cudaStream_t st); \

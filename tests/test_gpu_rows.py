@@ -44,6 +44,18 @@ def test_few_rows_identical(wts, M, d):
         assert torch.equal(wts.pairwise_dtw(gb), wts.pairwise_dtw(gb, o))
 
 
+@pytest.mark.parametrize("M", [1, 5, 127, 129, 300])
+def test_few_rows_identical_l2(wts, M):
+    rng = np.random.default_rng(M)
+    for d, integer in ((1, True), (3, False), (9, False)):
+        gb, draw = _batch(wts, rng, [1, 7, 8, 9, 31, 32, 33, 40, 200], d, integer)
+        B = torch.from_numpy(draw(M).astype(np.float32)).cuda()
+        a, o = wts.options(cost_kind=1), wts.options(cost_kind=1, rows_per_thread=16)
+        for x, y in zip(wts.dtw_align(B, gb, a, wts.Workspace()), wts.dtw_align(B, gb, o, wts.Workspace())):
+            assert torch.equal(x, y)
+        assert torch.equal(wts.pairwise_dtw(gb, a), wts.pairwise_dtw(gb, o))
+
+
 def test_overflowing_costs_identical(wts):
     """Finite samples whose squared differences overflow: every cost is +inf and
     ties decide, with few rows as with many."""
