@@ -85,7 +85,8 @@ typedef struct wts_options {
                                       are few), 32 if d <= 2 and else 16 with dir_mode = 1, 16 with a band; with the
                                       l2 norm 4, 16 for the score, Sub-DTW, a band and dir_mode = 1.  Results do not depend on it.  A workspace too small for that choice
                                       but large enough for 32 / 16 rows is accepted and runs those.  Soft-DTW does
-                                      not use it: 8 rows per lane, 4 under a band narrower than 0.45 */
+                                      not use it: 8 rows per lane, 4 under a band narrower than 0.45 or (R kept,
+                                      no band) for few and short pairs */
     int32_t warps_per_block;       /* 0 = 4; 1..4 */
     int32_t max_blocks;            /* 0 = as many as are resident at once (persistent grid); else a cap */
     int32_t keep_batch_order;      /* 0 = schedule the longest pairs first; 1 = batch order */

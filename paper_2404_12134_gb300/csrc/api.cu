@@ -135,8 +135,8 @@ int check_opt(const wts_options* opt, int D)
 }
 
 // Layout of the workspace for one call (host side; mirrors the setup kernel).
-// fixed_rows: rows per lane 32 / 16 by the channel count where the options name
-// none, instead of the choice by the launch's size (rows.cuh).
+// fixed_rows: rows per lane 32 / 16 by the channel count (soft-DTW: 8) where the
+// options name none, instead of the choice by the launch's size.
 int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L, bool fixed_rows = false)
 {
     int rc = check_batch(Y, false);
@@ -169,7 +169,7 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     }
     if (op == kOpSoft) {
         if (D > 8) return fail(WTS_EINVAL, "soft-DTW supports d <= 8 (got %d)", Y->d);
-        L->R = soft_rows(D);          // fixed by the channel count (registers)
+        L->R = fixed_rows || (opt && (opt->band > 0 || opt->dir_mode)) ? 8 : soft_rows(M, Y->T);
     }
     if (opt && opt->band > 0) {
         if (op != kOpSoft) {
@@ -1079,7 +1079,7 @@ int softdtw_forward(const float* B, int64_t M, const wts_batch* Y, float gamma, 
                     void* workspace, size_t workspace_bytes, void* stream, float* value)
 {
     Layout L;
-    int rc = compute_layout(kOpSoft, M, Y, opt, &L);
+    int rc = call_layout(kOpSoft, M, Y, opt, workspace_bytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if ((rc = check_gamma(gamma))) return rc;
@@ -1107,7 +1107,7 @@ int softdtw_backward(const float* B, int64_t M, const wts_batch* Y, float gamma,
                      float* grad_B)
 {
     Layout L;
-    int rc = compute_layout(kOpSoft, M, Y, opt, &L);
+    int rc = call_layout(kOpSoft, M, Y, opt, workspace_bytes, &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if ((rc = check_gamma(gamma))) return rc;
@@ -1214,7 +1214,8 @@ int wts_softdtw_barycenter_adam(float* B, int64_t M, const wts_batch* Y, float g
                                 void* workspace, size_t workspace_bytes, void* stream, float* values)
 {
     Layout L;
-    int rc = compute_layout(kOpSoft, M, Y, opt, &L);
+    const size_t extra_bytes = Y && M > 0 ? adam_extra_bytes(M, Y) : 0;
+    int rc = call_layout(kOpSoft, M, Y, opt, workspace_bytes - std::min(workspace_bytes, extra_bytes), &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if ((rc = check_gamma(gamma))) return rc;
@@ -1222,7 +1223,7 @@ int wts_softdtw_barycenter_adam(float* B, int64_t M, const wts_batch* Y, float g
     if (steps < 0) return fail(WTS_EINVAL, "steps must be >= 0");
     if (!(beta1 >= 0.f && beta1 < 1.f && beta2 >= 0.f && beta2 < 1.f && eps > 0.f))
         return fail(WTS_EINVAL, "need 0 <= beta < 1 and eps > 0");
-    const size_t need = L.total + adam_extra_bytes(M, Y);
+    const size_t need = L.total + extra_bytes;
     if (!workspace || ((uintptr_t)workspace & 255) != 0) return fail(WTS_EINVAL, "workspace must be 256-byte aligned");
     if (workspace_bytes < need) return fail(WTS_ENOMEM, "workspace has %zu bytes, needs %zu", workspace_bytes, need);
     cudaStream_t st = (cudaStream_t)stream;
@@ -1738,12 +1739,13 @@ int wts_softdtw_barycenter_lbfgs(float* B, int64_t M, const wts_batch* Y, float 
                                  int32_t* n_eval, int32_t* reason)
 {
     Layout L;
-    int rc = compute_layout(kOpSoft, M, Y, opt, &L);
+    const size_t extra_bytes = Y && M > 0 ? lbfgs_extra_bytes(M, Y) : 0;
+    int rc = call_layout(kOpSoft, M, Y, opt, workspace_bytes - std::min(workspace_bytes, extra_bytes), &L);
     if (rc) return rc;
     if ((rc = check_batch(Y, true))) return rc;
     if ((rc = check_gamma(gamma))) return rc;
     if (!B) return fail(WTS_EINVAL, "B must not be NULL");
-    const size_t need = L.total + lbfgs_extra_bytes(M, Y);
+    const size_t need = L.total + extra_bytes;
     if (!workspace || ((uintptr_t)workspace & 255) != 0) return fail(WTS_EINVAL, "workspace must be 256-byte aligned");
     if (workspace_bytes < need) return fail(WTS_ENOMEM, "workspace has %zu bytes, needs %zu", workspace_bytes, need);
     SoftObjective o;

@@ -858,11 +858,12 @@ cudaError_t launch_dbr(const SoftParams& p, int grid, int block, cudaStream_t st
     return run(soft_kernel<D, R, BWD, BANDED, COST, FUSED>());
 }
 
-// 8 rows per lane, or 4 under a narrow band (kSoftNarrowBand)
+// 8 rows per lane, or 4 under a narrow band (kSoftNarrowBand) or with R kept and
+// few warps (soft_rows)
 template <int D, bool BWD, bool BANDED, int COST, bool FUSED = false>
 cudaError_t launch_db(const SoftParams& p, int grid, int block, cudaStream_t st)
 {
-    if constexpr (BANDED) {
+    if constexpr (BANDED || !FUSED) {
         if (p.rows == 4) return launch_dbr<D, 4, BWD, BANDED, COST, FUSED>(p, grid, block, st);
     }
     return launch_dbr<D, 8, BWD, BANDED, COST, FUSED>(p, grid, block, st);
@@ -895,7 +896,7 @@ int occ_dbr(int block)
 template <int D, bool BWD, bool BANDED, int COST, bool FUSED = false>
 int occ_db(int block, int rows)
 {
-    if constexpr (BANDED) {
+    if constexpr (BANDED || !FUSED) {
         if (rows == 4) return occ_dbr<D, 4, BWD, BANDED, COST, FUSED>(block);
     }
     return occ_dbr<D, 8, BWD, BANDED, COST, FUSED>(block);

@@ -46,14 +46,29 @@ struct SoftParams {
     int skip_handoff;        // fault injection (tests): producers do not write hand-off rows
     int banded;              // pairs carry a Sakoe-Chiba band (PairDesc::band_bound); items run band-major
     int cost_kind;           // LocalCost
-    int rows;                // rows per lane R: 8, or 4 under a narrow band
+    int rows;                // rows per lane R: 8, or 4 (soft_rows, kSoftNarrowBand)
     int m_aligned;           // the prototype's M is a multiple of the rows per lane (every lane's rows
                              // lie all inside the matrix or all past it)
 };
 
-// Rows held per lane by the soft-DTW kernels (8 for every padded channel
-// count: measured best against 4 and 16).
-inline int soft_rows(int /*D*/) { return 8; }
+// Rows held per lane by the soft-DTW kernels without a band, R kept: 8 (measured
+// best against 4 and 16 with the warps of a full GPU), or 4 while the bands of 8
+// rows (256 prototype rows each) are at most kSoftFewBands, about five warps per
+// four schedulers, where a warp waits on the chain down its rows.  Measured,
+// forward + backward in us, 8 against 4 rows:
+//   16 x 1.1k x 6 ch    520 + 1004 /  432 +  651      (80 bands)
+//   64 x 3.0k x 1 ch   1323 + 1929 / 1186 + 1661     (768)
+//   64 x 3.0k x 8 ch   1710 + 2986 / 1587 + 2882     (768)
+//   32 x 8.0k x 8 ch   4707 + 8189 / 5579 + 10828   (1,024)
+//   64 x 8.0k x 1 ch   4434 + 6567 / 5182 + 8450    (2,048)
+// Prototypes over kSoftFewM rows keep 8, so that a long batch's workspaces with
+// R kept and with column checkpoints (8 rows always) differ by R alone.
+constexpr int kSoftFewBands = 768;
+constexpr int64_t kSoftFewM = 8192;
+inline int soft_rows(int64_t M, int T)
+{
+    return M <= kSoftFewM && T * cdiv(M, 256) <= kSoftFewBands ? 4 : 8;
+}
 // Under a Sakoe-Chiba band narrower than this fraction the soft-DTW passes
 // run 4 rows per lane: the band's lower edge is a chain of row bands, each
 // starting when the one above has covered its first 32 R + 62 columns, so

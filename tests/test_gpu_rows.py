@@ -75,6 +75,25 @@ def test_overflowing_costs_identical(wts):
         assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("cost", [0, 1])
+@pytest.mark.parametrize("d", [1, 3, 8])
+@pytest.mark.parametrize("M", [1, 3, 4, 127, 128, 129, 257, 600])
+def test_soft_few_rows_identical(wts, M, d, cost):
+    """Four rows (R kept, few pairs) against the checkpointed form, which holds
+    eight: values and gradient bit for bit."""
+    rng = np.random.default_rng(M + d)
+    gb, draw = _batch(wts, rng, [1, 2, 8, 31, 32, 33, 64, 65, 300], d, False)
+    B = torch.from_numpy(draw(M).astype(np.float32)).cuda()
+    got = []
+    for mode in (0, 1):
+        o, ws = wts.options(cost_kind=cost, dir_mode=mode), wts.Workspace()
+        v = wts.softdtw_forward(B, gb, 0.5, o, ws)
+        got.append((v, wts.softdtw_backward(B, gb, 0.5, None, o, ws)))
+        assert wts.read_status(ws.buf) == 0
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("op", ["score", "align"])
 def test_workspace_of_the_fixed_rows_is_accepted(wts, op):
     rng = np.random.default_rng(6)
