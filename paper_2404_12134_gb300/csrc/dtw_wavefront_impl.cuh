@@ -110,6 +110,13 @@ constexpr int kSlot = 4;     // u64 words after a warp's ring: its band's column
 
 constexpr int kSignD = 4;
 
+// Steps of the inner loop unrolled.  Four where a step is short (8 rows), and for
+// cost + |pi| up to four channels (uneven scoring, 1,000 cycles x 3 ch: wavefront
+// 143.5 -> 137.6 ms); two else: four of the long steps run the warps of a
+// scheduler out of the instruction cache (batched DBA, 6 ch: 68.7 -> 74.1 ms).
+template <int D, int R, int MODE>
+constexpr int kUnroll = R == 8 || (R == 16 && MODE == kModePlen && D <= 4) ? 4 : 2;
+
 // c[k] for a k known only at run time, by a binary tree of selects on the bits
 // of k (R - 1 selects, no local memory)
 template <int R>
@@ -470,7 +477,7 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
         auto chunk = [&](auto track) {
             constexpr bool TRACK = decltype(track)::value;
             if (full) {
-#pragma unroll (R == 8 ? 4 : 2)
+#pragma unroll (kUnroll<D, R, MODE>)
                 for (int u = 0; u < 32; ++u) st.template step<true, false, TRACK>(slot, u, lane, N, top);
             } else {
                 const int n = min(32, s_end - s0);
