@@ -360,23 +360,9 @@ int prepare(const Layout& L, char* ws, const float* B, const wts_batch* Y, const
 {
     cudaError_t e = cudaMemsetAsync(ws + L.off_hdr, 0, sizeof(WsHeader), st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(workspace header)");
-    // hand-off rows start as NaN: a slot is valid once its producer wrote it
-    if (L.hbuf_bytes) {
-        e = cudaMemsetAsync(ws + L.off_hbuf, 0xFF, L.hbuf_bytes, st);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(hand-off rows)");
-    }
-    // every sample must be finite (Sec. 3.1 removes missing values first): a
-    // non-finite one sets the status and abort words, and every kernel of the
-    // call then leaves at once
     DevInfo di;
     int rc = device_info(&di);
     if (rc) return rc;
-    {
-        Prof pr("setup", st);
-        e = launch_check_finite(B, B ? L.M * L.d : 0, Y->data, Y->offsets_host[Y->T] * Y->d,
-                                reinterpret_cast<WsHeader*>(ws + L.off_hdr), di.sms, st);
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "input check launch");
     SetupParams sp{};
     sp.op = L.op;
     sp.T = L.T;
@@ -395,12 +381,24 @@ int prepare(const Layout& L, char* ws, const float* B, const wts_batch* Y, const
     sp.group_bands = L.group_bands;
     sp.band = opt ? opt->band : 0.0;
     sp.store_pairs = L.store_pairs;
+    // every sample must be finite (Sec. 3.1 removes missing values first): a
+    // non-finite one sets the status and abort words, and every kernel of the
+    // call then leaves at once; hand-off rows start as NaN: a slot is valid once
+    // its producer wrote it
+    PrepParams pp{};
+    pp.a = B;
+    pp.na = B ? L.M * L.d : 0;
+    pp.b = Y->data;
+    pp.nb = Y->offsets_host[Y->T] * Y->d;
+    pp.hdr = reinterpret_cast<WsHeader*>(ws + L.off_hdr);
+    pp.fill = ws + L.off_hbuf;
+    pp.fill_bytes = L.hbuf_bytes;
     {
         Prof pr("setup", st);
-        launch_setup(sp, st);
+        pr.kernels = pp.fill_bytes > kPrepFillMax ? 2 : 1;
+        e = launch_prep(sp, pp, di.sms, st);
     }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "setup kernel launch");
+    if (e != cudaSuccess) return cuda_fail(e, "preparation launch");
     return WTS_OK;
 }
 

@@ -102,13 +102,27 @@ __host__ __device__ inline int64_t band_bound_of(double band, int64_t M, int64_t
     return (int64_t)floor(band * (double)M * (double)N);
 }
 
-void launch_setup(const SetupParams& sp, cudaStream_t st);
+// The rest of the preparation: scan a[0..na) and b[0..nb) (either may be null)
+// for a non-finite value (NaN or +-inf, Sec. 3.1 removes missing values before
+// alignment) - if one is found, hdr->status = kDevBadInput and hdr->abort = 1, so
+// that every kernel of the call leaves before doing any work - and fill
+// `fill_bytes` (a multiple of 4) at `fill` (16-byte aligned) with 0xFF.
+struct PrepParams {
+    const float* a;
+    int64_t na;
+    const float* b;
+    int64_t nb;
+    WsHeader* hdr;
+    void* fill;
+    size_t fill_bytes;
+};
 
-// Scan a[0..na) and b[0..nb) (either may be null) for a non-finite value (NaN
-// or +-inf, Sec. 3.1 removes missing values before alignment); if one is
-// found, set hdr->status = kDevBadInput and hdr->abort = 1, so that every
-// kernel of the call leaves before doing any work.  sms sizes the grid.
-cudaError_t launch_check_finite(const float* a, int64_t na, const float* b, int64_t nb, WsHeader* hdr, int sms,
-                                cudaStream_t st);
+// Up to this many bytes of hand-off rows it is one launch; above, a memset and two
+// kernels: the calls are long then, and rows filled by the kernel cost the passes
+// that follow more than the launches do (64 x 10k soft-DTW, 98 MB of rows: a
+// training step 15.2 -> 15.6 ms).
+constexpr size_t kPrepFillMax = 4u << 20;
+// hdr must be zero before it (stream order); sms sizes the grid.
+cudaError_t launch_prep(const SetupParams& sp, const PrepParams& pp, int sms, cudaStream_t st);
 
 }  // namespace wts
