@@ -42,6 +42,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase)
 // Row i's range is [jlo(i), jhi(i)]: jhi when the walk enters the row, jlo
 // when it leaves it (Definition "Alignment path": monotone, so each row's
 // columns are contiguous).
+// Bound by the walk's chain of dependent instructions (about 5 cycles each, one
+// warp per walk): 45 of them per run in the unchecked loop; 200 paths of 25k in 13
+// segments 0.67 ms (0.97 with the cell's read before its run's), 16 of 1.1k 65 us.
 template <int R>
 __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
 {

@@ -4,7 +4,7 @@
 //
 // The recursion, the lane skew, the local cost and the work list are those of
 // dtw_wavefront_impl.cuh (results are the same bit for bit).  What differs:
-//  - two or four rows per lane, so a step is short and a pair has many bands;
+//  - four rows per lane, so a step is short and a pair has many bands;
 //  - steps run in blocks of eight without a branch, at a band's two ends too
 //    (lanes outside the matrix keep their state by selects), every address an
 //    offset from the block's, the samples read a step ahead;
@@ -13,6 +13,10 @@
 //  - a code bit is the sign of m - v, shifted into the word (one subtraction on
 //    the FMA pipe and one funnel shift, where a comparison to a mask and its OR
 //    are three ALU instructions).
+// Measured (one pair, cost + |pi|): a step of 128 rows 62 ns at one channel, 83 at
+// nine, bands 66 steps apart; 1.1k x 1.1k x 1 ch 102 us against 121 with 8 rows per
+// lane and 265 with 32; Sub-DTW windows of 16k x 32k x 9 ch 6.35 -> 3.5 ms.  Bound
+// by dependent latencies: about 28 instructions a step at 3.3 cycles each.
 #pragma once
 
 #include "dtw_wavefront_impl.cuh"
@@ -32,6 +36,7 @@ __device__ __forceinline__ void sts64(uint32_t a, u64 v)
 {
     asm volatile("st.shared.b64 [%0], %1;" :: "r"(a), "l"(v) : "memory");
 }
+
 template <int D, int R, int MODE, int COST>
 struct Lean {
     static constexpr int Q = R / 2;

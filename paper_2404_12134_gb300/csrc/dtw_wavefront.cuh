@@ -40,7 +40,7 @@ struct DPParams {
     int skip_handoff;        // fault injection (tests): producers do not write hand-off rows
     int banded;              // pairs carry a Sakoe-Chiba band (PairDesc::band_bound); R = 16 only;
                              // items then run band-major (every pair's band 0, then band 1, ...)
-    int cost_kind;           // LocalCost; kCostL2 runs with R = 16 only
+    int cost_kind;           // LocalCost; kCostL2 runs with R = 16, or 4 (codes and cost, no band)
     int group_pairs;         // > 0: the work list takes pairs in groups of this many, band-major
                              // within a group; 0: pair after pair
     int group_bands;         // the most bands of a pair: the items per pair of a grouped list
