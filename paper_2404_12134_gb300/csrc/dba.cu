@@ -1,12 +1,12 @@
 // Backtrack of the tie-rule path, DBA averaging, and initial barycenters.
 #include "dba.cuh"
+#include "walk_window.h"
 
 namespace wts {
 
 namespace {
 
 constexpr int kBtWarps = 2;      // warps per backtrack CTA
-constexpr int kBtWords = 4096;   // 16 KB of direction words cached per warp
 constexpr long long kBtSpin = 1ll << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -48,10 +48,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase)
 template <int R>
 __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
 {
-    constexpr int W = R >= 16 ? R / 16 : 1;         // words per (word row, lane)
-    constexpr int SPW = R >= 16 ? 1 : 32 / (2 * R); // steps per word row
-    constexpr int LOG_R = R == 4 ? 2 : (R == 8 ? 3 : (R == 16 ? 4 : 5));
-    constexpr int kBtRows = kBtWords / (32 * W);    // word rows of one band in the window
+    using Win = WalkWindow<R>;
+    constexpr int W = Win::W, SPW = Win::SPW, LOG_R = Win::LOG_R, kBtRows = Win::ROWS;
     __shared__ __align__(128) uint32_t win_all[kBtWarps][kBtWords];
     __shared__ __align__(8) uint64_t bars[kBtWarps];
     const int lane = threadIdx.x & 31;
@@ -177,15 +175,16 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
             // away from the window's and the rows' ends: the same runs without a check
             // (in a loop of its own: a warp walking alone is bound by the chain of
             // dependent instructions, about 5 cycles each)
-            const int fi = max(b << (LOG_R + 5), i_lo + 1) + 16;
-            if (!mergeable && i >= fi && j >= 17 && j + ((i >> LOG_R) & 31) >= wlo * SPW + 21) {
-                const uint32_t* win0 = win - wlo * 32 * W;
+            const int floor = max(b << (LOG_R + 5), i_lo + 1);
+            const int first = wlo * SPW;             // the window's first step; jw: columns from there
+            int jw = j - first;
+            if (!mergeable && Win::inside(i, jw, first, floor)) {
                 int taken = 0;
                 do {
-                    const int iu = i - u_i, ju = j - u_j;
+                    const int iu = i - u_i, ju = jw - u_j;
                     const int tt = (iu >> LOG_R) & 31;
                     const int ss = ju + tt;
-                    const uint32_t* wp = win0 + ((ss / SPW) * 32 + tt) * W;
+                    const uint32_t* wp = win + Win::word(ss, tt);
                     const int kk = iu & (R - 1);
                     // "not diag" and "not up" of the cell at fixed places of x
                     uint32_t x;
@@ -200,13 +199,14 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
                     const int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
                     const int di = base != 24, dj = base != 16;
                     if (di && lane >= base && lane < base + run) {
-                        jlo[iu] = ju;
-                        jhi[iu - 1] = ju - dj;
+                        jlo[iu] = first + ju;
+                        jhi[iu - 1] = first + ju - dj;
                     }
                     i -= di ? run : 0;
-                    j -= dj ? run : 0;
+                    jw -= dj ? run : 0;
                     taken += run;
-                } while (i >= fi && j >= 17 && j + ((i >> LOG_R) & 31) >= wlo * SPW + 21);
+                } while (Win::inside(i, jw, first, floor));
+                j = first + jw;
                 len += taken - 1;
                 continue;
             }
@@ -222,10 +222,10 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
             const int iu = i - u_i, ju = j - u_j;
             const int tt = (iu >> LOG_R) & 31;
             const int ss = ju + tt;
-            const bool here = iu >= (b << (LOG_R + 5)) && ju >= 0 && ss >= wlo * SPW;
+            const bool here = iu >= (b << (LOG_R + 5)) && ju >= 0 && ss >= first;
             // cell (iu, ju) of the window: lane t = (iu mod BR) / R, row k = iu
             // mod R, step s = ju + t
-            const uint32_t* wp = win + (here ? ((ss / SPW - wlo) * 32 + tt) * W : 0);
+            const uint32_t* wp = win + (here ? Win::word(ss - first, tt) : 0);
             const int kk = iu & (R - 1);
             uint32_t nd, nu;
             if (R == 4) {
