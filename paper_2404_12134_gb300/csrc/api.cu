@@ -17,6 +17,7 @@
 #include "plan.cuh"
 #include "rows.cuh"
 #include "softdtw.cuh"
+#include "work_list.h"
 
 namespace wts {
 int run_probe(int which, double* ops_per_s);
@@ -457,8 +458,8 @@ int launch_dp(int mode, const Layout& L, const DPParams& p0, const wts_options* 
     // 16 such cycles 43.5 -> 41.8 ms).  Under a band every pair's band b comes before
     // any band b + 1 (one group).
     const int64_t nb = p.recompute ? p.band_cnt : L.max_bands;
-    if ((int64_t)L.P * nb < ((int64_t)1 << 31)) {
-        const int64_t warps = (int64_t)grid * (block / 32);
+    const int64_t warps = (int64_t)grid * (block / 32);
+    if (grouped_list_fits(L.P, nb, warps)) {
         p.group_pairs = p.banded ? L.P : (int)std::max<int64_t>(1, std::min<int64_t>(L.P, warps / nb));
         p.group_bands = (int)nb;
         if (!p.recompute) p.n_items = (int)(L.P * nb);
