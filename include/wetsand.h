@@ -83,7 +83,10 @@ typedef struct wts_options {
                                       0 = the library's choice: for anomaly_score, dtw_align, dba_iterate and the
                                       pairwise matrix by the launch's size (4, 8, 16 or 32; few rows while the warps
                                       are few), 32 if d <= 2 and else 16 with dir_mode = 1, 16 with a band; with the
-                                      l2 norm 4, 16 for the score, Sub-DTW, a band and dir_mode = 1.  Results do not depend on it.  A workspace too small for that choice
+                                      l2 norm 4, 16 for the score, Sub-DTW, a band and dir_mode = 1.  Results do
+                                      not depend on it.  The choice by size adds at most 16 GiB to the workspace
+                                      that 32 / 16 rows need, and nothing past 64 GiB in all (those rows run then).
+                                      A workspace too small for that choice
                                       but large enough for 32 / 16 rows is accepted and runs those.  Soft-DTW does
                                       not use it: 8 rows per lane, 4 under a band narrower than 0.45 or (R kept,
                                       no band) for few and short pairs */

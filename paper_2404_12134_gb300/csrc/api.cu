@@ -138,7 +138,7 @@ int check_opt(const wts_options* opt, int D)
 // Layout of the workspace for one call (host side; mirrors the setup kernel).
 // fixed_rows: rows per lane 32 / 16 by the channel count (soft-DTW: 8) where the
 // options name none, instead of the choice by the launch's size.
-int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L, bool fixed_rows = false)
+int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L, bool fixed_rows)
 {
     int rc = check_batch(Y, false);
     if (rc) return rc;
@@ -171,6 +171,7 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     if (op == kOpSoft) {
         if (D > 8) return fail(WTS_EINVAL, "soft-DTW supports d <= 8 (got %d)", Y->d);
         L->R = fixed_rows || (opt && (opt->band > 0 || opt->dir_mode)) ? 8 : soft_rows(M, Y->T);
+        L->rows_by_size = L->R != 8;
     }
     if (opt && opt->band > 0) {
         if (op != kOpSoft) {
@@ -195,6 +196,7 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     // (checkpointed codes count their memory in bands, so they keep the rows)
     if (!fixed_rows && (op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) &&
         !(opt && (opt->rows_per_thread || opt->band > 0 || opt->dir_mode)) && !(op == kOpScore && L->cost_kind)) {
+        const int fixed = L->R;
         if (L->cost_kind == WTS_COST_L2) {
             // four rows at every size: the square roots outweigh a step's fixed
             // work, and sixteen rows of them spill (ns of a step at full issue, 4
@@ -210,6 +212,7 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
             }
             L->R = load.rows(D, op == kOpScore ? kRowPlen : (op == kOpPairwise ? kRowCost : kRowCodes), L->R);
         }
+        L->rows_by_size = L->R != fixed;
     }
     L->BR = 32 * L->R;
     L->M = M;
@@ -321,6 +324,25 @@ int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt
     return WTS_OK;
 }
 
+// Fewer rows per lane mean more hand-off rows (one per band, for every pair at
+// once: with the l2 norm four times those of sixteen rows).  The choice by size
+// may cost up to kRowsRoom more than the fixed rows' layout and none more past
+// kRowsWhole, a quarter of the memory: a batch that fitted the GPU with the fixed
+// rows still does (the l2 pairwise matrix of 200 x 24.5k x 6 ch: 92 GB with
+// sixteen rows, 373 GB with four).
+constexpr size_t kRowsRoom = (size_t)16 << 30, kRowsWhole = (size_t)64 << 30;
+
+int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L)
+{
+    const int rc = layout_with(op, M, Y, opt, L, false);
+    if (rc == WTS_OK && !(L->rows_by_size && L->total > kRowsRoom)) return rc;
+    Layout F;
+    if (layout_with(op, M, Y, opt, &F, true) != WTS_OK) return rc;
+    // (rc: more items than a list holds, with few rows only)
+    if (rc || (L->total > F.total && (L->total > kRowsWhole || L->total - F.total > kRowsRoom))) *L = F;
+    return ok();
+}
+
 int check_ws(const Layout& L, const void* ws, size_t bytes)
 {
     if (!ws) return fail(WTS_EINVAL, "workspace is NULL");
@@ -337,7 +359,7 @@ int call_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, s
     int rc = compute_layout(op, M, Y, opt, L);
     if (rc || bytes >= L->total) return rc;
     Layout F;
-    if (compute_layout(op, M, Y, opt, &F, true) == WTS_OK && bytes >= F.total) *L = F;
+    if (layout_with(op, M, Y, opt, &F, true) == WTS_OK && bytes >= F.total) *L = F;
     return ok();
 }
 
