@@ -283,8 +283,8 @@ int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, L
     L->hbuf_bytes = (size_t)h * (op == kOpScore ? 8 : 4);
     // four rows per lane: the same hand-off area for the score and the paths,
     // so that one workspace of a small batch serves both
-    const size_t hbuf_room = op != kOpSubdtw && op != kOpSoft && L->R == 4 && !L->cost_kind ? (size_t)h * 8
-                                                                                            : L->hbuf_bytes;
+    const bool shared_room = op == kOpScore || op == kOpAlign || op == kOpDba;
+    const size_t hbuf_room = shared_room && L->R == 4 && !L->cost_kind ? (size_t)h * 8 : L->hbuf_bytes;
     L->ebuf_bytes = op == kOpSoft ? (size_t)h * 16 : 0;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off = align256(off + bytes); return at; };

@@ -55,3 +55,16 @@ def test_small_batches_take_the_larger_workspace(lib):
         m = 0 if op == _abi.OP_PAIRWISE else M
         assert _size(lib, op, m, [M] * T, d, cost_kind=cost_kind) > _size(
             lib, op, m, [M] * T, d, cost_kind=cost_kind, rows_per_thread=16 if d > 2 or cost_kind else 32)
+
+
+def test_pairwise_hand_off_slots_hold_the_cost_alone(lib):
+    """Four bytes a slot for the pairwise matrix, at every row count (only the score
+    counts path cells beside the cost)."""
+    T, n, d = 12, 6000, 3
+    bands = -(-n // 128)
+    got = _size(lib, _abi.OP_PAIRWISE, 0, [n] * T, d)
+    eight = _size(lib, _abi.OP_PAIRWISE, 0, [n] * T, d, rows_per_thread=8)
+    pairs = T * (T - 1) // 2
+    slots4, slots8 = pairs * (bands - 1) * n, pairs * (-(-n // 256) - 1) * n
+    assert got > eight                         # four rows are the choice here
+    assert abs((got - eight) - 4 * (slots4 - slots8)) <= 1024
