@@ -86,8 +86,8 @@ typedef struct wts_options {
                                       l2 norm 4, 16 for the score, Sub-DTW, a band and dir_mode = 1.  Results do
                                       not depend on it.  The choice by size adds at most 16 GiB to the workspace
                                       that 32 / 16 rows need, and nothing past 64 GiB in all (those rows run then).
-                                      A workspace too small for that choice
-                                      but large enough for 32 / 16 rows is accepted and runs those.  Soft-DTW does
+                                      A workspace too small for that choice (one sized for a larger batch, say)
+                                      but large enough for another row count is accepted and runs that.  Soft-DTW does
                                       not use it: 8 rows per lane, 4 under a band narrower than 0.45 or (R kept,
                                       no band) for few and short pairs */
     int32_t warps_per_block;       /* 0 = 4; 1..4 */

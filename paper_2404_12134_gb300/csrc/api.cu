@@ -136,9 +136,11 @@ int check_opt(const wts_options* opt, int D)
 }
 
 // Layout of the workspace for one call (host side; mirrors the setup kernel).
-// fixed_rows: rows per lane 32 / 16 by the channel count (soft-DTW: 8) where the
-// options name none, instead of the choice by the launch's size.
-int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L, bool fixed_rows)
+// rows: the rows per lane where neither the options nor the form name them: the
+// choice by the launch's size, the fixed rows (32 / 16 by the channel count,
+// soft-DTW 8), or a count that the form's kernels hold.
+constexpr int kRowsBySize = 0, kRowsFixed = -1;
+int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L, int rows)
 {
     int rc = check_batch(Y, false);
     if (rc) return rc;
@@ -170,7 +172,11 @@ int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, L
     }
     if (op == kOpSoft) {
         if (D > 8) return fail(WTS_EINVAL, "soft-DTW supports d <= 8 (got %d)", Y->d);
-        L->R = fixed_rows || (opt && (opt->band > 0 || opt->dir_mode)) ? 8 : soft_rows(M, Y->T);
+        L->R = 8;
+        if (!(opt && (opt->band > 0 || opt->dir_mode))) {
+            if (rows != kRowsFixed) L->R = rows == kRowsBySize ? soft_rows(M, Y->T) : rows;
+            L->rows_open = true;
+        }
         L->rows_by_size = L->R != 8;
     }
     if (opt && opt->band > 0) {
@@ -194,10 +200,13 @@ int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, L
     }
     const int64_t* o = Y->offsets_host;
     // (checkpointed codes count their memory in bands, so they keep the rows)
-    if (!fixed_rows && (op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) &&
+    if ((op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) &&
         !(opt && (opt->rows_per_thread || opt->band > 0 || opt->dir_mode)) && !(op == kOpScore && L->cost_kind)) {
         const int fixed = L->R;
-        if (L->cost_kind == WTS_COST_L2) {
+        L->rows_open = true;
+        if (rows != kRowsBySize) {
+            if (rows != kRowsFixed) L->R = rows;
+        } else if (L->cost_kind == WTS_COST_L2) {
             // four rows at every size: the square roots outweigh a step's fixed
             // work, and sixteen rows of them spill (ns of a step at full issue, 4
             // against 16 rows: d = 1 66 / 288, d = 6 98 / 468, d = 16 188 / 2136;
@@ -334,10 +343,10 @@ constexpr size_t kRowsRoom = (size_t)16 << 30, kRowsWhole = (size_t)64 << 30;
 
 int compute_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, Layout* L)
 {
-    const int rc = layout_with(op, M, Y, opt, L, false);
+    const int rc = layout_with(op, M, Y, opt, L, kRowsBySize);
     if (rc == WTS_OK && !(L->rows_by_size && L->total > kRowsRoom)) return rc;
     Layout F;
-    if (layout_with(op, M, Y, opt, &F, true) != WTS_OK) return rc;
+    if (layout_with(op, M, Y, opt, &F, kRowsFixed) != WTS_OK) return rc;
     // (rc: more items than a list holds, with few rows only)
     if (rc || (L->total > F.total && (L->total > kRowsWhole || L->total - F.total > kRowsRoom))) *L = F;
     return ok();
@@ -351,15 +360,23 @@ int check_ws(const Layout& L, const void* ws, size_t bytes)
     return WTS_OK;
 }
 
-// The layout that a call runs with in the workspace it was given: a workspace
-// sized for another batch (a longer one's is reused for shorter ones) may hold
-// the fixed rows' layout only, and then those run.
+// The layout that a call runs with in the workspace it was given.  A workspace
+// sized for another batch (a larger one's serves a part of it) may hold other rows
+// per lane than this call's choice alone: the larger batch's choice, or the fixed
+// rows.  Any that fit give the same results.
 int call_layout(int op, int64_t M, const wts_batch* Y, const wts_options* opt, size_t bytes, Layout* L)
 {
     int rc = compute_layout(op, M, Y, opt, L);
-    if (rc || bytes >= L->total) return rc;
-    Layout F;
-    if (layout_with(op, M, Y, opt, &F, true) == WTS_OK && bytes >= F.total) *L = F;
+    if (rc || bytes >= L->total || !L->rows_open) return rc;
+    for (int rows : {kRowsFixed, 8, 16, 32, 4}) {
+        if ((op == kOpSoft && rows > 8) || (op != kOpSoft && L->cost_kind && (rows == 8 || rows == 32)) ||
+            (rows == 32 && L->D > 3))
+            continue;
+        Layout F;
+        if (layout_with(op, M, Y, opt, &F, rows) != WTS_OK || bytes < F.total) continue;
+        *L = F;
+        break;
+    }
     return ok();
 }
 

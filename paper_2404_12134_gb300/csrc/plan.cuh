@@ -51,6 +51,7 @@ struct Layout {
     int T = 0;            // cycles in the batch
     int P = 0;            // alignment problems (T, or T(T-1)/2 for pairwise)
     int d = 0, D = 0, R = 0, BR = 0;
+    bool rows_open = false;      // neither the options nor the form name R
     bool rows_by_size = false;   // R is the choice by the launch's size, other than the fixed rows
     int64_t M = 0;        // prototype length (shared-prototype ops)
     int64_t n_items = 0;  // total (pair, band) items
