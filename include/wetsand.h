@@ -139,7 +139,10 @@ typedef struct wts_options {
                                       the checkpoints take about 0.3 bytes per cell, and the memory left
                                       can hold R of some pairs instead of recomputing it.  Non-zero with
                                       any other operation or mode is WTS_EINVAL. */
-    int32_t reserved[3];
+    int32_t rows_by_size;          /* 1: rows per lane by the launch's size as with rows_per_thread = 0, which then
+                                      names the rows to run where that choice does not apply or fit
+                                      (what wts_autotune returns when the choice by size is the fastest) */
+    int32_t reserved[2];
 } wts_options;
 
 /* Values of wts_options.cost_kind. */
@@ -430,8 +433,9 @@ int wts_softdtw_barycenter_adam(float* B, int64_t M, const wts_batch* Y, float g
  * the wavefront for operation op (WTS_OP_ANOMALY_SCORE, WTS_OP_DTW_ALIGN or
  * WTS_OP_DBA_ITERATE) on this batch by timing each candidate that fits in the
  * given workspace (one warm-up and the best of two timed passes each, CUDA
- * events on `stream`; synchronises it; the default shape is kept unless another
- * is more than 1 % faster).  Results are cached per (op, d, M, T, total
+ * events on `stream`; synchronises it; the default, rows by the launch's size, is
+ * kept unless another is more than 1 % faster, and returned as rows_by_size = 1
+ * where it is not one of 8, 16 and 32 rows alone).  Results are cached per (op, d, M, T, total
  * length); a cached answer costs nothing.  best: out (host); best_ms: out
  * (host, may be NULL), the wavefront time of the chosen options.
  */

@@ -56,7 +56,8 @@ class wts_options(ctypes.Structure):
         ("cost_kind", ctypes.c_int32),
         ("score_via_codes", ctypes.c_int32),
         ("store_pairs", ctypes.c_int32),
-        ("reserved", ctypes.c_int32 * 3),
+        ("rows_by_size", ctypes.c_int32),
+        ("reserved", ctypes.c_int32 * 2),
     ]
 
 

@@ -59,7 +59,7 @@ class Batch:
 
 def options(rows_per_thread=0, warps_per_block=0, max_blocks=0, keep_batch_order=0, dir_mode=0,
             ckpt_bands=0, spin_limit=0, fault_skip_handoff=0, band=0.0, cost_kind=0,
-            score_via_codes=0, store_pairs=0) -> wts_options:
+            score_via_codes=0, store_pairs=0, rows_by_size=0) -> wts_options:
     """Launch and method options (see wts_options in include/wetsand.h); band > 0
     is the Sakoe-Chiba width (Table I) for the DTW operations; cost_kind 1 takes
     the l2 norm as the local cost instead of its square (Sec. 3.2);
@@ -67,6 +67,7 @@ def options(rows_per_thread=0, warps_per_block=0, max_blocks=0, keep_batch_order
     store_pairs keeps R of the longest pairs in soft-DTW's checkpoint mode."""
     o = wts_options()
     o.store_pairs = store_pairs
+    o.rows_by_size = rows_by_size
     o.score_via_codes = score_via_codes
     o.band = float(band)
     o.cost_kind = cost_kind
@@ -408,7 +409,7 @@ def autotune(op: int, B: torch.Tensor, batch: Batch, ws: Workspace | None = None
     M = B.shape[0]
     forms = (0, 1) if op == _abi.OP_ANOMALY_SCORE else (0,)
     need = max(workspace_size(op, M, batch, options(rows_per_thread=r, score_via_codes=f))
-               for r in ((8, 16, 32) if batch.d <= 3 else (8, 16)) for f in forms)
+               for r in ((0, 8, 16, 32) if batch.d <= 3 else (0, 8, 16)) for f in forms)
     buf = _ws(ws, need)
     best = wts_options()
     ms = ctypes.c_float(0)

@@ -200,8 +200,9 @@ int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, L
     }
     const int64_t* o = Y->offsets_host;
     // (checkpointed codes count their memory in bands, so they keep the rows)
-    if ((op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) &&
-        !(opt && (opt->rows_per_thread || opt->band > 0 || opt->dir_mode)) && !(op == kOpScore && L->cost_kind)) {
+    const bool named = opt && opt->rows_per_thread && opt->rows_by_size != 1;
+    if ((op == kOpScore || op == kOpAlign || op == kOpDba || op == kOpPairwise) && !named &&
+        !(opt && (opt->band > 0 || opt->dir_mode)) && !(op == kOpScore && L->cost_kind)) {
         const int fixed = L->R;
         L->rows_open = true;
         if (rows != kRowsBySize) {
@@ -1306,7 +1307,8 @@ int wts_autotune(int op, const float* B, int64_t M, const wts_batch* Y, void* wo
         wts_options o{};
         o.score_via_codes = 1;
         Layout Lc;
-        codes_fit = compute_layout(kop, M, Y, &o, &Lc) == WTS_OK && check_ws(Lc, workspace, workspace_bytes) == WTS_OK;
+        codes_fit = call_layout(kop, M, Y, &o, workspace_bytes, &Lc) == WTS_OK &&
+                    check_ws(Lc, workspace, workspace_bytes) == WTS_OK;
     }
     static std::mutex mu;
     static std::map<std::tuple<int, int, int64_t, int, int64_t, int>, std::pair<wts_options, float>> cache;
@@ -1323,27 +1325,31 @@ int wts_autotune(int op, const float* B, int64_t M, const wts_batch* Y, void* wo
     cudaStream_t st = (cudaStream_t)stream;
     const int D = pick_D(Y->d);
     std::vector<wts_options> cands;
-    // the default shape first: another candidate must beat it by more than 1 %
-    for (int R : {D <= 2 ? 32 : 16, D <= 2 ? 16 : 32, 8}) {
-        if (R == 32 && D > 3) continue;
-        for (int wpb : {4, 2, 1}) {
-            wts_options o{};
-            o.rows_per_thread = R;
-            o.warps_per_block = wpb;
-            cands.push_back(o);
-        }
-    }
+    const int fixed = pick_R(D, nullptr), other = fixed == 32 ? 16 : 32;
+    auto add = [&](int R, int wpb, int by_size, int via_codes) {
+        if (R == 32 && D > 3) return;
+        wts_options o{};
+        o.rows_per_thread = R;
+        o.warps_per_block = wpb;
+        o.rows_by_size = by_size;
+        o.score_via_codes = via_codes;
+        Layout L;
+        // rows by size only where they differ from the fixed ones (which follow)
+        if (by_size && (call_layout(kop, M, Y, &o, workspace_bytes, &L) != WTS_OK || !L.rows_by_size)) return;
+        cands.push_back(o);
+    };
+    // the default shape first (rows by the launch's size): another candidate must
+    // beat it by more than 1 %
+    for (int wpb : {4, 2, 1}) add(fixed, wpb, 1, 0);
+    for (int R : {fixed, other, 8})
+        for (int wpb : {4, 2, 1}) add(R, wpb, 0, 0);
     // the score through stored codes and the walk (when the workspace holds
-    // the codes): the two row counts of the code-writing DP, 4 warps per block
-    if (kop == kOpScore)
-        for (int R : {D <= 2 ? 32 : 16, D <= 2 ? 16 : 32}) {
-            if (R == 32 && D > 3) continue;
-            wts_options o{};
-            o.rows_per_thread = R;
-            o.warps_per_block = 4;
-            o.score_via_codes = 1;
-            cands.push_back(o);
-        }
+    // the codes): the row counts of the code-writing DP, 4 warps per block
+    if (kop == kOpScore) {
+        add(fixed, 4, 1, 1);
+        add(fixed, 4, 0, 1);
+        add(other, 4, 0, 1);
+    }
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess)
         return fail(WTS_ECUDA, "cudaEventCreate");
@@ -1370,7 +1376,7 @@ int wts_autotune(int op, const float* B, int64_t M, const wts_batch* Y, void* wo
     };
     for (const wts_options& o : cands) {
         Layout L;
-        if (compute_layout(kop, M, Y, &o, &L) != WTS_OK) continue;
+        if (call_layout(kop, M, Y, &o, workspace_bytes, &L) != WTS_OK) continue;
         if (check_ws(L, workspace, workspace_bytes) != WTS_OK) continue;
         float t_min = 1e30f;
         for (int rep = 0; rep < 3; ++rep) {             // first run warms up, best of two
