@@ -208,13 +208,7 @@ int anomaly_score(const float* B, int64_t M, const wts_batch* Y, const wts_optio
  * visits each row on one contiguous run of columns), and |pi_k| = sum_i
  * (jhi - jlo + 1).
  *   cost [T], plen [T]           out (either may be NULL)
- *   jlo  [T][M], jhi [T][M]      out (int32); with every code stored
- *                                (dir_mode 0) the walk reads the jhi values
- *                                found there on entry as guesses of where
- *                                the path enters rows 256 to 2048 apart (a repeated
- *                                call on the same arrays walks faster); any
- *                                contents are safe and the result does not
- *                                depend on them
+ *   jlo  [T][M], jhi [T][M]      out (int32; contents on entry are not read)
  * A 2-bit predecessor code per cell is kept in the workspace (M*N_k/4 bytes
  * per cycle, plus a skew margin); wts_workspace_size(WTS_OP_DTW_ALIGN, ...).
  */
@@ -355,11 +349,8 @@ int wts_softdtw_barycenter_lbfgs(float* B, int64_t M, const wts_batch* Y, float 
  *   B_in [M][d], B_out [M][d] (must not alias B_in)
  *   counts [M] out (may be NULL), cost_before: one double, out (may be NULL),
  *   cost [T] out (may be NULL): DTW(B_in, Y_k)
- * Workspace: wts_workspace_size(WTS_OP_DBA_ITERATE, ...).  The paths are kept
- * in the workspace; with every code stored (dir_mode 0) the next call on the
- * same workspace and batch starts its walk from them as guesses (faster
- * between DBA iterations, whose paths move little); any workspace contents
- * give the same result.
+ * Workspace: wts_workspace_size(WTS_OP_DBA_ITERATE, ...); its contents on
+ * entry are not read.
  */
 int dba_iterate(const float* B_in, float* B_out, int64_t M, const wts_batch* Y, const wts_options* opt,
                 void* workspace, size_t workspace_bytes, void* stream,

@@ -238,8 +238,7 @@ def noalloc_status() -> int:
 def dtw_align(B: torch.Tensor, batch: Batch, opts=None, ws: Workspace | None = None,
               jlo: torch.Tensor | None = None, jhi: torch.Tensor | None = None):
     """DTW and tie-rule path per cycle: (cost [T], plen [T], jlo [T, M], jhi [T, M]).
-    jlo / jhi may be given (int32 [T, M], written in place); the ranges they
-    hold on entry serve the walk as guesses (the previous call's paths)."""
+    jlo / jhi may be given (int32 [T, M], written in place)."""
     B = _check_B(B, batch.d)
     M = B.shape[0]
     lib = _abi.load()

@@ -308,12 +308,17 @@ int layout_with(int op, int64_t M, const wts_batch* Y, const wts_options* opt, L
         if (opt && opt->dir_mode == 1) {
             L->group_bands = opt->ckpt_bands ? opt->ckpt_bands : 16;
             L->off_btstate = take((size_t)L->T * sizeof(int32_t));
-            L->nseg = (int)cdiv(std::min<int64_t>(M, (int64_t)L->group_bands * L->BR),
-                                bt_seg_rows((int64_t)L->group_bands * L->BR));
-            L->off_seg = take((size_t)L->P * L->nseg * 4 * sizeof(int32_t));
-        } else if (op != kOpSubdtw) {
-            L->nseg = (int)cdiv(M, bt_seg_rows(M));
-            L->off_seg = take((size_t)L->P * L->nseg * 4 * sizeof(int32_t));
+        }
+        if (op != kOpSubdtw) {
+            // the walk's segments: of all rows, or of a group's
+            const int64_t group = L->group_bands ? std::min<int64_t>(M, (int64_t)L->group_bands * L->BR) : M;
+            L->lead_rows = bt_lead_rows(M);
+            if (L->group_bands) L->lead_rows = std::min(L->lead_rows, (int)cdiv(group, 4));
+            L->seg_rows = bt_seg_rows(group, L->P, L->lead_rows);
+            L->nseg = (int)cdiv(group, L->seg_rows);
+            // (room for any number of pairs up to this one)
+            const int64_t room = std::min((int64_t)L->P * cdiv(group, 128), std::max<int64_t>(L->P, kBtResident));
+            L->off_seg = take((size_t)room * 4 * sizeof(int32_t));
         }
     }
     if (op == kOpDba) {
@@ -513,18 +518,14 @@ int launch_dp(int mode, const Layout& L, const DPParams& p0, const wts_options* 
     return WTS_OK;
 }
 
-// The rounds of a segmented walk and its last kernel.
+// A segmented walk: all segments at once, those entered elsewhere again, |pi|.
 cudaError_t segmented_walk(BTParams bt, cudaStream_t st)
 {
     Prof pr("backtrack", st);
-    pr.kernels = bt.nseg + 1;
-    for (int r = 0; r < bt.nseg; ++r) {
-        bt.round = r;
-        const cudaError_t e = launch_backtrack(bt, st);
-        if (e != cudaSuccess) return e;
-    }
-    bt.round = bt.nseg - 1;
-    return launch_backtrack_seg_final(bt, st);
+    pr.kernels = 3;
+    cudaError_t e = cudaSuccess;
+    for (bt.join = 0; bt.join < 2 && e == cudaSuccess; ++bt.join) e = launch_backtrack(bt, st);
+    return e == cudaSuccess ? launch_backtrack_seg_final(bt, st) : e;
 }
 
 // Shared body of dtw_align and dba_iterate: directions + backtrack.
@@ -552,11 +553,10 @@ int align_into(const Layout& L, char* ws, const float* B, const wts_batch* Y, co
         if (rc) return rc;
         bt.band_lo = 0;
         bt.band_hi = (int)cdiv(L.M, L.BR);
-        // segmented walk: nseg rounds (a round only re-walks the segments
-        // whose start changed), then |pi| from the ranges; a single segment
-        // is one plain walk per pair
+        // a single segment is one plain walk per pair
         bt.nseg = L.nseg > 1 ? L.nseg : 0;
-        bt.seg_rows = bt_seg_rows(L.M);
+        bt.seg_rows = L.seg_rows;
+        bt.lead_rows = L.lead_rows;
         bt.seg = reinterpret_cast<int32_t*>(ws + L.off_seg);
         bt.first = 1;
         if (bt.nseg == 0) {
@@ -579,7 +579,8 @@ int align_into(const Layout& L, char* ws, const float* B, const wts_batch* Y, co
     bt.state = reinterpret_cast<int32_t*>(ws + L.off_btstate);
     bt.seg = reinterpret_cast<int32_t*>(ws + L.off_seg);
     bt.nseg = L.nseg;
-    bt.seg_rows = bt_seg_rows((int64_t)G * L.BR);
+    bt.seg_rows = L.seg_rows;
+    bt.lead_rows = L.lead_rows;
     for (int hi = nb; hi > 0; hi -= G) {
         const int lo = hi - G > 0 ? hi - G : 0;
         DPParams r = p;

@@ -8,6 +8,7 @@ namespace {
 
 constexpr int kBtWarps = 2;      // warps per backtrack CTA
 constexpr long long kBtSpin = 1ll << 24;
+constexpr int kBtBurst = 64;     // rows a second walk takes unchecked between looks for the first
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
@@ -43,8 +44,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase)
 // when it leaves it (Definition "Alignment path": monotone, so each row's
 // columns are contiguous).
 // Bound by the walk's chain of dependent instructions (about 5 cycles each, one
-// warp per walk): 45 of them per run in the unchecked loop; 200 paths of 25k in 13
-// segments 0.67 ms (0.97 with the cell's read before its run's), 16 of 1.1k 65 us.
+// warp per walk): 45 of them per run in the unchecked loop; 16 paths of 1.1k in 9
+// segments 70 us (one walk a path 235), 200 of 25k in 9 1.00 ms, 32 of 110k in 14
+// checkpointed groups 7.3 ms (22.3), whatever the range arrays hold.
 template <int R>
 __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
 {
@@ -71,234 +73,259 @@ __global__ void __launch_bounds__(32 * kBtWarps) backtrack_kernel(BTParams p)
     const int u_i = g_i ? u : 0, u_j = g_j ? u : 0;
     uint32_t phase = 0;
     bool failed = false;
-    const int units = p.nseg > 0 ? p.P * p.nseg : p.P;
+    const bool seg = p.nseg > 0;
+    const int units = seg && !p.join ? p.P * p.nseg : p.P;
     for (int un = blockIdx.x * kBtWarps + wid; un < units && !failed; un += gridDim.x * kBtWarps) {
-        const int q = p.nseg > 0 ? un / p.nseg : un;
+        const int q = seg && !p.join ? un / p.nseg : un;
         const PairDesc pd = p.pairs[q];
         const int N = pd.N;
         int32_t* jlo = p.jlo + (int64_t)pd.out * p.M;
         int32_t* jhi = p.jhi + (int64_t)pd.out * p.M;
-        int i, j, len;
         const int row_lo = p.band_lo * 32 * R, row_hi = min((int64_t)pd.M, (int64_t)p.band_hi * 32 * R);
-        int i_lo = row_lo;
-        int32_t* sg = p.nseg > 0 ? p.seg + 4 * (int64_t)un : nullptr;
-        const int cur = p.round & 1;
-        bool mergeable = false, merged = false;
-        int prev_exit = -1;
-        if (p.nseg > 0) {
-            // segment sk: rows [row_lo + sk * seg_rows, top]; the last one holds the group's last row
-            const int sk = un - q * p.nseg;
-            i_lo = row_lo + sk * p.seg_rows;
-            if (i_lo >= row_hi) continue;
-            const int top = min(row_hi, i_lo + p.seg_rows) - 1;
-            int start;
-            if (top == row_hi - 1) {
-                if (p.round > 0) {                   // walked from the path's entry in round 0
-                    if (lane == 0) sg[1 + cur] = sg[2 - cur];
-                    continue;
-                }
-                start = p.first ? N - 1 : p.state[q];
-            } else if (p.round == 0) {
-                // a guess: the column this row was entered at by the previous
-                // walk of this pair (the ranges of an earlier call on the same
-                // arrays; any value is safe), else the diagonal
-                start = jhi[top];
-                if (start < 0 || start >= N) start = (int)((int64_t)top * (N - 1) / max(pd.M - 1, 1));
-            } else {
-                start = p.seg[4 * (int64_t)(un + 1) + 2 - cur];     // exit of the segment above, last round
-                if (start == sg[0]) {                // unchanged: the walk recorded stands
-                    if (lane == 0) sg[1 + cur] = sg[2 - cur];
-                    continue;
-                }
-            }
-            if (start < 0 || start >= N) {           // the segment above failed
-                if (lane == 0) { sg[0] = start; sg[1 + cur] = -1; sg[3] = 1; }
-                continue;
-            }
-            // A re-walk (round > 0) stops where it enters the previous walk of
-            // this segment, whose ranges the arrays hold: from a shared cell
-            // the walks are the same.  Row top of that walk is [jlo(top), old
-            // start].
-            mergeable = p.round > 0 && sg[3] == 0;
-            prev_exit = sg[2 - cur];
-            if (mergeable && jlo[top] <= start && start <= sg[0]) {
-                __syncwarp();
-                if (lane == 0) { jhi[top] = start; sg[0] = start; sg[1 + cur] = prev_exit; }
-                continue;
-            }
-            i = top; j = start; len = 0;
-            if (lane == 0) { jhi[i] = j; sg[0] = start; }
-        } else {
-            i = pd.M - 1; j = p.subseq ? p.bstar[pd.out] : N - 1; len = 0;
-            if (j < 0 || j >= N) {                    // b* is not a column of this cycle: no walk
-                if (lane == 0) {
-                    if (p.astar) p.astar[pd.out] = -1;
-                    if (p.plen) p.plen[pd.out] = -1;
-                }
-                continue;
-            }
-            if (lane == 0) jhi[i] = j;
+        // the segments of this warp: one, or (join) all but the topmost from the top down
+        int sk = 0, sk_end = 0, above = 0;
+        if (seg && !p.join) {
+            sk = sk_end = un - q * p.nseg;
+            if (row_lo + sk * p.seg_rows >= row_hi) continue;
+        } else if (seg) {
+            sk = (row_hi - row_lo + p.seg_rows - 1) / p.seg_rows - 1;
+            above = p.seg[4 * ((int64_t)q * p.nseg + sk) + 1];
+            --sk;
         }
-        int band = -1, wlo = 0, whi = -1;           // word rows in the window
-        bool left_group = false;
-        for (;;) {
-            ++len;
-            if (i == 0 && j == 0) break;
-            const int b = i >> (LOG_R + 5);
-            const int row = (j + ((i >> LOG_R) & 31)) / SPW;     // word row of step s = j + t
-            if (b != band || row < wlo || row > whi) {
-                band = b;
-                whi = row;
-                wlo = max(0, row - kBtRows + 1);
-                const uint32_t* src = p.dirs + pd.dir_off + (int64_t)(b - p.band_lo) * band_dir_words(N, R) +
-                                      (int64_t)wlo * 32 * W;
-                const uint32_t bytes = (uint32_t)(whi - wlo + 1) * 32 * W * 4;
-                __syncwarp();
-                if (lane == 0) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                                 :: "r"(smem_u32(bar)), "r"(bytes) : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 :: "r"(smem_u32(win)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-                }
-                const bool ok = mbar_wait(bar, phase);
-                phase ^= 1u;
-                if (!ok) {
-                    // the copy did not land in time: give up on this pair,
-                    // wait (bounded) for the copy still in flight, stop
-                    mbar_wait(bar, phase ^ 1u);
-                    len = -1;
-                    failed = true;
-                    break;
-                }
-            }
-            // away from the window's and the rows' ends: the same runs without a check
-            // (in a loop of its own: a warp walking alone is bound by the chain of
-            // dependent instructions, about 5 cycles each)
-            const int floor = max(b << (LOG_R + 5), i_lo + 1);
-            const int first = wlo * SPW;             // the window's first step; jw: columns from there
-            int jw = j - first;
-            if (!mergeable && Win::inside(i, jw, first, floor)) {
-                int taken = 0;
-                do {
-                    const int iu = i - u_i, ju = jw - u_j;
-                    const int tt = (iu >> LOG_R) & 31;
-                    const int ss = ju + tt;
-                    const uint32_t* wp = win + Win::word(ss, tt);
-                    const int kk = iu & (R - 1);
-                    // "not diag" and "not up" of the cell at fixed places of x
-                    uint32_t x;
-                    if (R == 32) x = ((wp[0] << kk) & 0x80000000u) | (((wp[W - 1] << kk) >> 1) & 0x40000000u);
-                    else x = wp[0] << (R == 4 ? (ss % SPW) * 2 * R + 2 * kk : R == 8 ? kk + 16 - (ss & 1) * 16 : kk);
-                    constexpr uint32_t ND = R == 16 ? 0x8000u : (R == 8 ? 0x800000u : 0x80000000u);
-                    constexpr uint32_t NU = R == 16 || R == 8 ? 0x80000000u : 0x40000000u;
-                    const uint32_t mask = group == 0 ? ND : (ND | NU);
-                    const uint32_t want = group == 0 ? 0u : (group == 1 ? ND : (ND | NU));
-                    const uint32_t votes = __ballot_sync(FULL, (x & mask) == want);
-                    const int base = __ffs(votes & 0x01010001u) - 1;
-                    const int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
-                    const int di = base != 24, dj = base != 16;
-                    if (di && lane >= base && lane < base + run) {
-                        jlo[iu] = first + ju;
-                        jhi[iu - 1] = first + ju - dj;
+        for (; sk >= sk_end && !failed; --sk) {
+            int i, j, len = 0;
+            int i_lo = row_lo;
+            int32_t* sg = seg ? p.seg + 4 * ((int64_t)q * p.nseg + sk) : nullptr;
+            bool mergeable = false, merged = false;
+            bool lead = false;               // above the segment: nothing is recorded
+            int old_exit = -1;
+            if (seg) {
+                // segment sk: rows [row_lo + sk * seg_rows, top]; the topmost one holds the group's last row
+                i_lo = row_lo + sk * p.seg_rows;
+                const int top = min(row_hi, i_lo + p.seg_rows) - 1;
+                if (!p.join) {
+                    // the path enters the group's last row at `entry` and ends at (0, 0):
+                    // from the line between them, lead_rows above the segment's top
+                    const int entry = p.first ? N - 1 : p.state[q];
+                    const int from = (int)min((int64_t)top + p.lead_rows, (int64_t)row_hi - 1);
+                    i = from;
+                    j = from == row_hi - 1 ? entry : (int)((int64_t)from * entry / (row_hi - 1));
+                    lead = from > top;
+                    if (entry < 0 || entry >= N) {       // the group above failed
+                        if (lane == 0) { sg[0] = -1; sg[1] = -1; sg[3] = 1; }
+                        continue;
                     }
-                    i -= di ? run : 0;
-                    jw -= dj ? run : 0;
-                    taken += run;
-                } while (Win::inside(i, jw, first, floor));
-                j = first + jw;
-                len += taken - 1;
-                continue;
-            }
-            // Runs: the lanes read ahead along all three kinds of move at once,
-            // 16 cells on the diagonal, 8 up, 8 left (lane u of a group the cell
-            // that u moves of its kind would reach); a lane agrees if its cell is
-            // in the window and codes the group's move and, past the first, the
-            // move is an ordinary one (not out of the grid, not out of the rows
-            // loaded).  The first lane of one group agrees, which is the cell's
-            // own move, and the lanes that agree after it are the run: the same
-            // walk as one cell at a time, with one shared-memory read and one
-            // vote per run (the read of the cell, then of its run, took two).
-            const int iu = i - u_i, ju = j - u_j;
-            const int tt = (iu >> LOG_R) & 31;
-            const int ss = ju + tt;
-            const bool here = iu >= (b << (LOG_R + 5)) && ju >= 0 && ss >= first;
-            // cell (iu, ju) of the window: lane t = (iu mod BR) / R, row k = iu
-            // mod R, step s = ju + t
-            const uint32_t* wp = win + (here ? Win::word(ss - first, tt) : 0);
-            const int kk = iu & (R - 1);
-            uint32_t nd, nu;
-            if (R == 4) {
-                const uint32_t w1 = wp[0] << ((ss % SPW) * 2 * R + 2 * kk);
-                nd = w1 >> 31;
-                nu = (w1 >> 30) & 1u;
-            } else {
-                const uint32_t w0 = R < 16 ? wp[0] >> ((ss % SPW) * 2 * R) : wp[0];
-                nd = (w0 >> (R - 1 - kk)) & 1u;
-                nu = R <= 16 ? (w0 >> (2 * R - 1 - kk)) & 1u : (wp[W - 1] >> (R - 1 - kk)) & 1u;
-            }
-            // codes: diag (nd = 0) moves up-left, up (nd = 1, nu = 0) moves up,
-            // left (nd = nu = 1) moves left
-            const int kind = nd == 0u ? 0 : (nu == 0u ? 1 : 2);
-            const bool agree = here && kind == group &&
-                               (u == 0 || ((!g_i || (iu > 0 && iu - 1 >= i_lo)) && (!g_j || ju > 0)));
-            const uint32_t votes = __ballot_sync(FULL, agree);
-            const int base = __ffs(votes & 0x01010001u) - 1;       // the group's first lane
-            const int di = base != 24, dj = base != 16;
-            // Sub-DTW: a move up from row 0 reaches the free start
-            if (p.subseq && i == 0 && di) break;
-            // a valid code matrix only moves left on row 0 and only up on
-            // column 0; anything else is reported as |pi| = -1
-            if ((i == 0 && di) || (j == 0 && dj)) { len = -1; break; }
-            int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
-            // a re-walk: does the move of c_u enter a row at a cell of the
-            // previous walk (read before this run's writes)?
-            const bool mine = lane >= base && lane < base + run && di;
-            uint32_t mv = 0u;
-            if (mergeable) {                         // warp-uniform
-                bool mg = false;
-                if (mine && iu - 1 >= i_lo) {
-                    const int je = ju - dj;
-                    mg = jlo[iu - 1] <= je && je <= jhi[iu - 1];
-                }
-                mv = __ballot_sync(FULL, mg);
-                if (mv) run = __ffs(mv) - base;      // up to and including the first such move
-            }
-            if (mine && lane < base + run) {
-                jlo[iu] = ju;
-                jhi[iu - 1] = ju - dj;
-            }
-            i -= run * di;
-            j -= run * dj;
-            len += run - 1;
-            if (mv) { merged = true; break; }
-            if (i < i_lo) { left_group = true; break; }    // the rest lies in bands not loaded
-        }
-        if (sg != nullptr) {
-            if (lane == 0) {
-                if (merged) {
-                    sg[1 + cur] = prev_exit;          // the rest is the previous walk's
+                    if (lead) i_lo = top + 1;
+                    if (lane == 0) {
+                        sg[0] = lead ? -1 : j;
+                        if (!lead) jhi[i] = j;
+                    }
                 } else {
-                    sg[1 + cur] = left_group ? j : -1;    // the path's column in the row below
+                    if (above == sg[0]) {                // the walk recorded stands
+                        above = sg[1];
+                        continue;
+                    }
+                    if (above < 0 || above >= N) {       // the segment above failed
+                        __syncwarp();
+                        if (lane == 0) { sg[0] = above; sg[1] = -1; sg[3] = 1; }
+                        above = -1;
+                        continue;
+                    }
+                    // A second walk stops where it enters the first one of this
+                    // segment, whose ranges the arrays hold: from a shared cell the
+                    // walks are the same.  Row top of the first is [jlo(top), its start].
+                    mergeable = sg[3] == 0;
+                    old_exit = sg[1];
+                    const bool at_top = mergeable && jlo[top] <= above && above <= sg[0];
+                    __syncwarp();
+                    if (lane == 0) { jhi[top] = above; sg[0] = above; }
+                    if (at_top) {
+                        above = old_exit;
+                        continue;
+                    }
+                    i = top; j = above;
+                }
+            } else {
+                i = pd.M - 1; j = p.subseq ? p.bstar[pd.out] : N - 1;
+                if (j < 0 || j >= N) {                    // b* is not a column of this cycle: no walk
+                    if (lane == 0) {
+                        if (p.astar) p.astar[pd.out] = -1;
+                        if (p.plen) p.plen[pd.out] = -1;
+                    }
+                    continue;
+                }
+                if (lane == 0) jhi[i] = j;
+            }
+            bool vote_next = false;                     // a second walk: after unchecked rows, a checked run
+            int band = -1, wlo = 0, whi = -1;           // word rows in the window
+            bool left_group = false;
+            for (;;) {
+                ++len;
+                if (i == 0 && j == 0) break;
+                const int b = i >> (LOG_R + 5);
+                const int row = (j + ((i >> LOG_R) & 31)) / SPW;     // word row of step s = j + t
+                if (b != band || row < wlo || row > whi) {
+                    band = b;
+                    whi = row;
+                    wlo = max(0, row - kBtRows + 1);
+                    const uint32_t* src = p.dirs + pd.dir_off + (int64_t)(b - p.band_lo) * band_dir_words(N, R) +
+                                          (int64_t)wlo * 32 * W;
+                    const uint32_t bytes = (uint32_t)(whi - wlo + 1) * 32 * W * 4;
+                    __syncwarp();
+                    if (lane == 0) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                                     :: "r"(smem_u32(bar)), "r"(bytes) : "memory");
+                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                     :: "r"(smem_u32(win)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+                    }
+                    const bool ok = mbar_wait(bar, phase);
+                    phase ^= 1u;
+                    if (!ok) {
+                        // the copy did not land in time: give up on this pair,
+                        // wait (bounded) for the copy still in flight, stop
+                        mbar_wait(bar, phase ^ 1u);
+                        len = -1;
+                        failed = true;
+                        break;
+                    }
+                }
+                // away from the window's and the rows' ends: the same runs without a check
+                // (in a loop of its own: a warp walking alone is bound by the chain of
+                // dependent instructions, about 5 cycles each)
+                // (a second walk: kBtBurst rows at a time, then a run that looks for the first walk)
+                int floor = max(b << (LOG_R + 5), i_lo + 1);
+                if (mergeable) floor = max(floor, i - kBtBurst);
+                const int first = wlo * SPW;             // the window's first step; jw: columns from there
+                int jw = j - first;
+                if (!vote_next && Win::inside(i, jw, first, floor)) {
+                    vote_next = mergeable;
+                    int taken = 0;
+                    do {
+                        const int iu = i - u_i, ju = jw - u_j;
+                        const int tt = (iu >> LOG_R) & 31;
+                        const int ss = ju + tt;
+                        const uint32_t* wp = win + Win::word(ss, tt);
+                        const int kk = iu & (R - 1);
+                        // "not diag" and "not up" of the cell at fixed places of x
+                        uint32_t x;
+                        if (R == 32) x = ((wp[0] << kk) & 0x80000000u) | (((wp[W - 1] << kk) >> 1) & 0x40000000u);
+                        else x = wp[0] << (R == 4 ? (ss % SPW) * 2 * R + 2 * kk : R == 8 ? kk + 16 - (ss & 1) * 16 : kk);
+                        constexpr uint32_t ND = R == 16 ? 0x8000u : (R == 8 ? 0x800000u : 0x80000000u);
+                        constexpr uint32_t NU = R == 16 || R == 8 ? 0x80000000u : 0x40000000u;
+                        const uint32_t mask = group == 0 ? ND : (ND | NU);
+                        const uint32_t want = group == 0 ? 0u : (group == 1 ? ND : (ND | NU));
+                        const uint32_t votes = __ballot_sync(FULL, (x & mask) == want);
+                        const int base = __ffs(votes & 0x01010001u) - 1;
+                        const int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
+                        const int di = base != 24, dj = base != 16;
+                        if (di && !lead && lane >= base && lane < base + run) {
+                            jlo[iu] = first + ju;
+                            jhi[iu - 1] = first + ju - dj;
+                        }
+                        i -= di ? run : 0;
+                        jw -= dj ? run : 0;
+                        taken += run;
+                    } while (Win::inside(i, jw, first, floor));
+                    j = first + jw;
+                    len += taken - 1;
+                    continue;
+                }
+                vote_next = false;
+                // Runs: the lanes read ahead along all three kinds of move at once,
+                // 16 cells on the diagonal, 8 up, 8 left (lane u of a group the cell
+                // that u moves of its kind would reach); a lane agrees if its cell is
+                // in the window and codes the group's move and, past the first, the
+                // move is an ordinary one (not out of the grid, not out of the rows
+                // loaded).  The first lane of one group agrees, which is the cell's
+                // own move, and the lanes that agree after it are the run: the same
+                // walk as one cell at a time, with one shared-memory read and one
+                // vote per run (the read of the cell, then of its run, took two).
+                const int iu = i - u_i, ju = j - u_j;
+                const int tt = (iu >> LOG_R) & 31;
+                const int ss = ju + tt;
+                const bool here = iu >= (b << (LOG_R + 5)) && ju >= 0 && ss >= first;
+                // cell (iu, ju) of the window: lane t = (iu mod BR) / R, row k = iu
+                // mod R, step s = ju + t
+                const uint32_t* wp = win + (here ? Win::word(ss - first, tt) : 0);
+                const int kk = iu & (R - 1);
+                uint32_t nd, nu;
+                if (R == 4) {
+                    const uint32_t w1 = wp[0] << ((ss % SPW) * 2 * R + 2 * kk);
+                    nd = w1 >> 31;
+                    nu = (w1 >> 30) & 1u;
+                } else {
+                    const uint32_t w0 = R < 16 ? wp[0] >> ((ss % SPW) * 2 * R) : wp[0];
+                    nd = (w0 >> (R - 1 - kk)) & 1u;
+                    nu = R <= 16 ? (w0 >> (2 * R - 1 - kk)) & 1u : (wp[W - 1] >> (R - 1 - kk)) & 1u;
+                }
+                // codes: diag (nd = 0) moves up-left, up (nd = 1, nu = 0) moves up,
+                // left (nd = nu = 1) moves left
+                const int kind = nd == 0u ? 0 : (nu == 0u ? 1 : 2);
+                const bool agree = here && kind == group &&
+                                   (u == 0 || ((!g_i || (iu > 0 && iu - 1 >= i_lo)) && (!g_j || ju > 0)));
+                const uint32_t votes = __ballot_sync(FULL, agree);
+                const int base = __ffs(votes & 0x01010001u) - 1;       // the group's first lane
+                const int di = base != 24, dj = base != 16;
+                // Sub-DTW: a move up from row 0 reaches the free start
+                if (p.subseq && i == 0 && di) break;
+                // a valid code matrix only moves left on row 0 and only up on
+                // column 0; anything else is reported as |pi| = -1
+                if ((i == 0 && di) || (j == 0 && dj)) { len = -1; break; }
+                int run = __ffs(~((votes >> base) & (base == 0 ? 0xffffu : 0xffu))) - 1;
+                // a re-walk: does the move of c_u enter a row at a cell of the
+                // previous walk (read before this run's writes)?
+                const bool mine = lane >= base && lane < base + run && di;
+                uint32_t mv = 0u;
+                if (mergeable) {                         // warp-uniform
+                    bool mg = false;
+                    if (mine && iu - 1 >= i_lo) {
+                        const int je = ju - dj;
+                        mg = jlo[iu - 1] <= je && je <= jhi[iu - 1];
+                    }
+                    mv = __ballot_sync(FULL, mg);
+                    if (mv) run = __ffs(mv) - base;      // up to and including the first such move
+                }
+                if (mine && !lead && lane < base + run) {
+                    jlo[iu] = ju;
+                    jhi[iu - 1] = ju - dj;
+                }
+                i -= run * di;
+                j -= run * dj;
+                len += run - 1;
+                if (mv) { merged = true; break; }
+                if (i < i_lo) {
+                    if (!lead) { left_group = true; break; }   // the rest lies in bands not loaded
+                    // the segment's top row: from here on the walk is recorded
+                    lead = false;
+                    i_lo = row_lo + sk * p.seg_rows;
+                    if (lane == 0) { jhi[i] = j; sg[0] = j; }
+                }
+            }
+            if (seg) {
+                // the path's column in the row below (merged: the rest is the first walk's)
+                above = merged ? old_exit : (left_group ? j : -1);
+                if (lane == 0 && !merged) {
+                    sg[1] = above;
                     sg[3] = len < 0 ? 1 : 0;
                     if (!left_group && i == 0 && j == 0 && len > 0) jlo[0] = 0;
                 }
+                continue;
             }
-            continue;
-        }
-        if (lane == 0) {
-            if (p.subseq) {
-                if (len > 0) jlo[0] = j;
-                p.astar[pd.out] = len > 0 ? j : -1;
-            } else if (i == 0 && j == 0 && len > 0) {
-                jlo[0] = 0;
+            if (lane == 0) {
+                if (p.subseq) {
+                    if (len > 0) jlo[0] = j;
+                    p.astar[pd.out] = len > 0 ? j : -1;
+                } else if (i == 0 && j == 0 && len > 0) {
+                    jlo[0] = 0;
+                }
+                if (p.plen) p.plen[pd.out] = len;
             }
-            if (p.plen) p.plen[pd.out] = len;
         }
     }
 }
 
-// One warp per pair, after the last round of a segmented walk: the segments
+// One warp per pair, after the two launches of a segmented walk: the segments
 // must join up (each one's start = the exit of the one above) and none may
 // have failed; then |pi| = sum_i (jhi(i) - jlo(i) + 1), the cells of a monotone
 // path being row by row contiguous.
@@ -309,17 +336,16 @@ __global__ void __launch_bounds__(128) bt_seg_final_kernel(BTParams p)
     if (q >= p.P) return;
     if (p.hdr != nullptr && ld_volatile(&p.hdr->abort)) return;      // nothing was walked
     const PairDesc pd = p.pairs[q];
-    const int last = (p.round & 1);                  // exit slot of the last round
     const int rows = min((int64_t)pd.M, (int64_t)p.band_hi * 32 * p.R) - p.band_lo * 32 * p.R;
     const int nseg = (rows + p.seg_rows - 1) / p.seg_rows;
     bool bad = false;
     for (int k = lane; k < nseg; k += 32) {
         const int32_t* sg = p.seg + 4 * ((int64_t)q * p.nseg + k);
         if (sg[3] != 0) bad = true;
-        if (k + 1 < nseg && sg[0] != p.seg[4 * ((int64_t)q * p.nseg + k + 1) + 1 + last]) bad = true;
+        if (k + 1 < nseg && sg[0] != sg[4 + 1]) bad = true;
     }
     bad = __any_sync(FULL, bad);
-    if (p.state != nullptr && lane == 0) p.state[q] = bad ? -1 : p.seg[4 * (int64_t)q * p.nseg + 1 + last];
+    if (p.state != nullptr && lane == 0) p.state[q] = bad ? -1 : p.seg[4 * (int64_t)q * p.nseg + 1];
     if (p.band_lo > 0) return;                       // rows below are still to be walked
     const int32_t* jlo = p.jlo + (int64_t)pd.out * p.M;
     const int32_t* jhi = p.jhi + (int64_t)pd.out * p.M;
@@ -459,9 +485,10 @@ cudaError_t launch_backtrack(const BTParams& p, cudaStream_t st)
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int units = p.nseg > 0 ? p.P * p.nseg : p.P;
+    const bool by_segment = p.nseg > 0 && !p.join;
+    const int units = by_segment ? p.P * p.nseg : p.P;
     const int need = (units + kBtWarps - 1) / kBtWarps;
-    const int cap = (p.nseg > 0 ? 8 : 4) * sms;
+    const int cap = (by_segment ? 8 : 4) * sms;
     const int grid = need < cap ? need : cap;
     if (p.R == 4) backtrack_kernel<4><<<grid, 32 * kBtWarps, 0, st>>>(p);
     else if (p.R == 8) backtrack_kernel<8><<<grid, 32 * kBtWarps, 0, st>>>(p);

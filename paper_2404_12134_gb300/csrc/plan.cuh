@@ -63,7 +63,8 @@ struct Layout {
     int group_bands = 0;  // checkpoint mode: bands whose codes are recomputed at a time (0 = codes stored)
     int banded = 0;       // a Sakoe-Chiba band applies (the banded kernels run with R = 16)
     int cost_kind = 0;    // local cost: 0 squared l2, 1 the l2 norm (DTW kernels with R = 16)
-    int nseg = 0;         // segments of the segmented backtrack (codes stored, not Sub-DTW)
+    // the segmented backtrack (not Sub-DTW): segments, rows of one, rows walked above one
+    int nseg = 0, seg_rows = 0, lead_rows = 0;
     int soft_fused = 0;   // soft-DTW checkpoint mode without a band: column checkpoints, fused backward
     int store_pairs = 0;  // soft_fused: the first store_pairs pairs of the longest-first order keep R
     size_t off_seg = 0;
