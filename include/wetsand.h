@@ -386,7 +386,9 @@ int softdtw_forward(const float* B, int64_t M, const wts_batch* Y, float gamma, 
  * exp(((r(s) - r(i,j)) - delta(s))/gamma) e(s).  With g_k = lambda_k / m_k this
  * is the gradient of the barycenter objective Eq. 7.
  * The workspace must still hold the R written by softdtw_forward for the same
- * B, Y, gamma and options (the call may be repeated with other g).
+ * B, Y, gamma, options and workspace_bytes (the call may be repeated with other g).
+ * A workspace_bytes that leads to other rows per lane than the forward's raises the
+ * device status WTS_EINVAL (wts_read_status), and grad_B is not the gradient.
  *   grad_value [T] in (g_k), or NULL for Eq. 7's weights with lambda_k = 1:
  *   g_k = 1 / N_k (rounded to FP32, computed on the device);
  *   grad_B [M][d] out; the sum over k is in FP64, k ascending.

@@ -427,6 +427,7 @@ int prepare(const Layout& L, char* ws, const float* B, const wts_batch* Y, const
     sp.group_bands = L.group_bands;
     sp.band = opt ? opt->band : 0.0;
     sp.store_pairs = L.store_pairs;
+    sp.hdr = reinterpret_cast<WsHeader*>(ws + L.off_hdr);
     // every sample must be finite (Sec. 3.1 removes missing values first): a
     // non-finite one sets the status and abort words, and every kernel of the
     // call then leaves at once; hand-off rows start as NaN: a slot is valid once
@@ -1155,7 +1156,8 @@ int softdtw_backward(const float* B, int64_t M, const wts_batch* Y, float gamma,
     if ((rc = check_ws(L, workspace, workspace_bytes))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
-    cudaError_t e = cudaMemsetAsync(ws + L.off_hdr + offsetof(WsHeader, item_counter), 0, sizeof(int), st);
+    // (the rows per lane, so where R lies, depend on the workspace's size)
+    cudaError_t e = launch_softdtw_begin(reinterpret_cast<WsHeader*>(ws + L.off_hdr), L.R, st);
     if (e == cudaSuccess && L.ebuf_bytes) e = cudaMemsetAsync(ws + L.off_ebuf, 0xFF, L.ebuf_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(backward hand-off rows)");
     SoftParams p = soft_params(L, ws, gamma, opt);

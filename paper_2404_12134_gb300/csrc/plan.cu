@@ -52,6 +52,7 @@ __device__ void decode_pair(int p, int T, int* a, int* b)
 __device__ void build_work_list(const SetupParams& sp)
 {
     const int P = sp.P;
+    if (threadIdx.x == 0) sp.hdr->rows = sp.R;
     // pass 1: descriptors and storage offsets in pair order
     int64_t run_h = 0, run_d = 0, run_r = 0;
     for (int base = 0; base < P; base += kSetupThreads) {

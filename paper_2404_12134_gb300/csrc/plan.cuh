@@ -88,6 +88,7 @@ struct SetupParams {
     int group_bands;           // > 0: directions for only this many bands per pair (checkpoint mode)
     double band;               // Sakoe-Chiba width (0 = none): band_bound = floor(band * M * N)
     int store_pairs;           // soft-DTW column checkpoints: pairs of rank < store_pairs keep R instead
+    WsHeader* hdr;             // its `rows` is written
 };
 
 // Rank of pair p in the longest-first order (cells descending, ties by index),

@@ -949,6 +949,23 @@ int softdtw_max_blocks_per_sm(int D, int backward, int block, int banded, int co
     return 0;
 }
 
+namespace {
+__global__ void softdtw_begin_kernel(WsHeader* hdr, int rows)
+{
+    hdr->item_counter = 0;
+    if (hdr->rows != rows) {
+        hdr->status = kDevBadInput;
+        hdr->abort = 1;
+    }
+}
+}  // namespace
+
+cudaError_t launch_softdtw_begin(WsHeader* hdr, int rows, cudaStream_t st)
+{
+    softdtw_begin_kernel<<<1, 1, 0, st>>>(hdr, rows);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_softdtw_grad_reduce(const float* gpart, const float* g, const int64_t* offsets, int T, int64_t M,
                                        int d, float* grad_B, cudaStream_t st)
 {

@@ -83,6 +83,11 @@ cudaError_t launch_softdtw_bwd(int D, const SoftParams& p, int grid, int block, 
 int softdtw_max_blocks_per_sm(int D, int backward, int block, int banded = 0, int cost_kind = 0, int fused = 0,
                               int rows = 8);
 
+// Before a backward pass: the item cursor to zero; if the forward that filled the
+// workspace ran with other rows per lane (its workspace_bytes was another), R lies
+// elsewhere: status and abort are raised, and the pass leaves at once.
+cudaError_t launch_softdtw_begin(WsHeader* hdr, int rows, cudaStream_t st);
+
 // grad_B[i][c] = sum_k g[k] * gpart[k][i][c] (FP64 sum, k ascending); g == null
 // takes g[k] = 1 / N_k (Eq. 7 with lambda_k = 1) from the cycle offsets
 cudaError_t launch_softdtw_grad_reduce(const float* gpart, const float* g, const int64_t* offsets, int T, int64_t M,

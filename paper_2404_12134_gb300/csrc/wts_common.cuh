@@ -48,7 +48,8 @@ struct WsHeader {
     int item_counter;    // work-list cursor of the persistent kernels
     int abort;           // set with status so that waiting warps leave at once
     int timeout_where;   // which wait gave up (diagnostics)
-    int pad[60];
+    int rows;            // rows per lane of the layout that the call ran with
+    int pad[59];
 };
 
 __device__ __forceinline__ float inf_f() { return __int_as_float(0x7f800000); }
