@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(128, D <= 8 ? 3 : 2) dtw_lean_kernel(DPParams 
         if (item >= p.n_items) break;
         if (ld_volatile(&p.hdr->abort)) break;
         int q, band;
-        item_of(p, item, q, band);
+        item_of<false>(p, item, q, band);
         const PairDesc pd = p.pairs[p.order[q]];
         if (band < pd.nbands) lean_band<D, R, MODE, COST>(p, pd, band, lane, ring);
     }

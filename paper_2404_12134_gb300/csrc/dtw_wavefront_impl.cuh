@@ -104,18 +104,26 @@ __device__ __forceinline__ uint32_t ne_mask(float a, float b)
 // loads need no address arithmetic.
 constexpr int kRing = 164;
 __device__ __forceinline__ int ring_place(int s0) { return (s0 & 127) ? (s0 & 127) : 128; }
+// From seven channels on, but for nine, a step computes its own addresses (StepBand)
+// and the ring is the four chunks alone, without copies.
+template <int D>
+constexpr bool kPerStep = D > 6 && D != 9;
+template <int D>
+constexpr int kRingOf = kPerStep<D> ? 128 : kRing;
 constexpr int kSlot = 4;     // u64 words after a warp's ring: its band's columns and the band
 
 
 
 constexpr int kSignD = 4;
 
-// Steps of the inner loop unrolled.  Four where a step is short (8 rows), and for
-// cost + |pi| up to four channels (uneven scoring, 1,000 cycles x 3 ch: wavefront
-// 143.5 -> 137.6 ms); two else: four of the long steps run the warps of a
-// scheduler out of the instruction cache (batched DBA, 6 ch: 68.7 -> 74.1 ms).
-template <int D, int R, int MODE>
-constexpr int kUnroll = R == 8 || (R == 16 && MODE == kModePlen && D <= 4) ? 4 : 2;
+// Steps of the inner loop unrolled.  Four where a step is short (8 rows up to four
+// channels), and for cost + |pi| up to four channels (uneven scoring, 1,000 cycles x 3
+// ch: wavefront 143.5 -> 137.6 ms; under a band it costs, l2 100 x 6k x 3 ch 6.3 -> 7.1
+// ms); two else: four of the long steps run the warps of a scheduler out of the
+// instruction cache (batched DBA, 6 ch: 68.7 -> 74.1 ms; 8 rows, 6 ch, pairwise 24 of 6k
+// 5.2 -> 5.6 ms).
+template <int D, int R, int MODE, bool BANDED>
+constexpr int kUnroll = (R == 8 && D <= 4) || (R == 16 && MODE == kModePlen && D <= 4 && !BANDED) ? 4 : 2;
 
 // c[k] for a k known only at run time, by a binary tree of selects on the bits
 // of k (R - 1 selects, no local memory)
@@ -328,11 +336,129 @@ struct Band {
     }
 };
 
+// The step for wide samples (kPerStep): addresses from the step's number, code bits
+// by comparison, a Sub-DTW band's last row tracked behind a branch.  A chunk's
+// addresses, held beside 16 rows of 8 channels and more, and a second loop for the
+// tracked band cost these instances more than they save; with sixteen channels the
+// prototype rows spill, and a ring with copies takes the L1 that holds them (shared
+// memory of two blocks 130 -> 170 KB of the SM's 256).  Wavefront, 300 pairs of 6k (100 at 16
+// channels), 16 rows, per chunk / per step in ms: 8 channels codes 8.5 / 7.7, 16
+// channels codes 10.9 / 7.0, cost + |pi| 16.5 / 9.0, l2 checkpointed 50 / 23.6, Sub-DTW
+// l2 28 / 13.4, 12 channels 28 / 23.4.  At nine channels: codes 8.4 / 9.4.
+template <int D, int R, int MODE, bool BANDED, int COST>
+struct StepBand : Band<D, R, MODE, BANDED, COST> {
+    using B = Band<D, R, MODE, BANDED, COST>;
+    using B::CODES; using B::W; using B::Q;
+    using B::col; using B::dl; using B::cnt; using B::prev_up; using B::prev_upc; using B::topv; using B::topc;
+    using B::half; using B::kk; using B::best; using B::bestj; using B::cost_pair;
+    static constexpr int RING = kRingOf<D>;
+    bool track;
+
+    __device__ __forceinline__ void load_column(const u64* ring, int jc, u64* yy)
+    {
+        const u64* yr = ring + (jc & (RING - 1));
+#pragma unroll
+        for (int c = 0; c < D; ++c) yy[c] = yr[c * RING];
+    }
+
+    // One step: the lane's column j = s - lane (in range when FULLCHUNK), the value
+    // above its band's first row in lane u.
+    template <bool FULLCHUNK, bool MASK = false>
+    __device__ __forceinline__ void step_at(const u64* ring, int s, int u, int lane, int N, bool top, void* hcur,
+                                            uint32_t* dout)
+    {
+        const float INF = inf_f();
+        const float above = __shfl_up_sync(FULL, col[R - 1], 1);
+        const float tv = __shfl_sync(FULL, topv, u);
+        const float top_in = MODE == kModeSubDirs ? 0.f : INF;
+        const float up_in = lane == 0 ? (top ? top_in : tv) : above;
+        const float dg_in = prev_up;
+        prev_up = up_in;
+        int upc_in = 0, dgc_in = 0;
+        if (MODE == kModePlen) {
+            const int abovec = __shfl_up_sync(FULL, cnt[R - 1], 1);
+            const int tc = __shfl_sync(FULL, topc, u);
+            upc_in = lane == 0 ? tc : abovec;
+            dgc_in = prev_upc;
+            prev_upc = upc_in;
+        }
+        const int j = s - lane;
+        u64 yy[D];
+        load_column(ring, j + 1, yy);
+        uint32_t word = 0u;
+        const u64* slot = ring + D * RING;
+        bool valid = true;
+        int klo = 0, khi = R - 1;
+        if (!FULLCHUNK && !BANDED) valid = j >= 0 && j < N;
+        if (!FULLCHUNK && BANDED) {
+            const u64 cols = slot[0];
+            valid = j >= (int)(uint32_t)cols && j <= (int)(cols >> 32);
+            if (MASK) {
+                const u64 im = slot[1];
+                const int64_t bnd = (int64_t)slot[2];
+                const int i0 = (int)(uint32_t)im + lane * R;
+                const int64_t jm = (int64_t)j * (int64_t)(im >> 32);
+                klo = (int)max((int64_t)-1, ceil_div64(jm - bnd, N) - i0);
+                khi = (int)min((int64_t)R, floor_div64(jm + bnd, N) - i0);
+            }
+        }
+        if (FULLCHUNK || valid) {
+            float dg = dg_in, up = up_in;
+            int cdg = dgc_in, cup = upc_in;
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const float lf = col[k];
+                const float m = min3f(dg, up, lf);
+                float r = __fadd_rn(dl[k], m);
+                if (MASK && (k < klo || k > khi)) r = INF;     // outside the band
+                if (CODES) {
+                    word |= ne_mask(dg, m) & (1u << (R - 1 - k));
+                    word |= ne_mask(up, m) & (1u << (2 * R - 1 - k));
+                } else if (MODE == kModePlen) {
+                    const int cl = cnt[k];
+                    const int cn = 1 + (dg == m ? cdg : (up == m ? cup : cl));
+                    cdg = cl;
+                    cup = cn;
+                    cnt[k] = cn;
+                }
+                dg = lf;
+                up = r;
+                col[k] = r;
+                if (k & 1) cost_pair(yy, k >> 1);      // rows k-1, k of column j+1
+            }
+            if (MODE == kModeSubDirs && track) {
+                const float v = pick_row<R>(col, kk);
+                if (v < best) { best = v; bestj = j; }
+            }
+            if (lane == 31 && hcur != nullptr) {
+                if (MODE == kModePlen)
+                    __stcg(reinterpret_cast<u64*>(hcur) + j, pack2(col[R - 1], __int_as_float(cnt[R - 1])));
+                else
+                    __stcg(reinterpret_cast<float*>(hcur) + j, col[R - 1]);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) cost_pair(yy, q);
+        }
+        if (CODES) {
+            if (W == 0) {
+                if ((s & 1) == 0)
+                    half = word;
+                else
+                    __stcs(dout + (int64_t)(s >> 1) * 32 + lane, __byte_perm(half, word, 0x5410));
+            } else {
+                __stcs(dout + (int64_t)s * 32 + lane, word);
+            }
+        }
+    }
+};
+
 template <int D, int R, int MODE, bool BANDED, int COST>
 __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, int band, int lane, u64* ring)
 {
-    using BandT = Band<D, R, MODE, BANDED, COST>;
+    using BandT = std::conditional_t<kPerStep<D>, StepBand<D, R, MODE, BANDED, COST>, Band<D, R, MODE, BANDED, COST>>;
     constexpr int BR = BandT::BR;
+    constexpr int RING = kRingOf<D>;
     constexpr int W = BandT::W;
     const int M = pd.M, N = pd.N, d = p.d;
     const int i0 = band * BR + lane * R;
@@ -358,6 +484,7 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     st.topv = INF;
     st.topc = 0;
     st.half = 0u;
+    if constexpr (kPerStep<D>) st.track = MODE == kModeSubDirs && last;
     st.kk = M - 1 - i0;
     st.best = INF;
     st.bestj = 0;
@@ -378,7 +505,7 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
         if (!top) { jtop_lo = lo_of(r0 - 1); jtop_hi = hi_of(r0 - 1); }
         if (i0 < M) { full_lo = lo_of(min(i0 + R - 1, M - 1)); full_hi = hi_of(i0); }
     }
-    u64* slot = ring + D * kRing;
+    u64* slot = ring + D * RING;
     if (BANDED) {
         __syncwarp();
         if (lane == 0) {
@@ -418,9 +545,13 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     auto put_y = [&](int jj) {
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-            u64* row = ring + c * kRing;
+            u64* row = ring + c * RING;
             const u64 v = pack2(ynext[c], ynext[c]);
             const int i = jj & 127;
+            if (kPerStep<D>) {
+                row[i] = v;
+                continue;
+            }
             row[i < 32 ? i + 128 : i] = v;
             if (i < 36) row[i < 32 ? i : i + 128] = v;
         }
@@ -438,11 +569,14 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     load_y(s_begin + lane + 64);
     if (!top) tnext = load_t(s_begin + lane);
     __syncwarp();
-    st.begin_chunk(ring, s_begin, lane, hcur, dout);
+    if constexpr (!kPerStep<D>) st.begin_chunk(ring, s_begin, lane, hcur, dout);
     {
         // local costs of the lane's first column (j = s_begin - lane)
         u64 yy[D];
-        st.load_samples(0, yy);
+        if constexpr (kPerStep<D>)
+            st.load_column(ring, s_begin - lane, yy);
+        else
+            st.load_samples(0, yy);
 #pragma unroll
         for (int q = 0; q < BandT::Q; ++q) st.cost_pair(yy, q);
     }
@@ -469,26 +603,37 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
                 tnext = load_t(jj + 32);
             }
         }
-        st.begin_chunk(ring, s0, lane, hcur, dout);
+        if constexpr (!kPerStep<D>) st.begin_chunk(ring, s0, lane, hcur, dout);
         // every lane in the band's columns and inside the band all chunk long
         const bool full = BANDED ? (s0 - 31 >= jlo_b && s0 + 31 <= jhi_b &&
                                     __all_sync(FULL, s0 - lane >= full_lo && s0 + 31 - lane <= full_hi))
                                  : (s0 >= 31 && s0 + 32 <= N);
-        auto chunk = [&](auto track) {
-            constexpr bool TRACK = decltype(track)::value;
+        if constexpr (kPerStep<D>) {
             if (full) {
-#pragma unroll (kUnroll<D, R, MODE>)
-                for (int u = 0; u < 32; ++u) st.template step<true, false, TRACK>(slot, u, lane, N, top);
+#pragma unroll 2
+                for (int u = 0; u < 32; ++u) st.template step_at<true>(ring, s0 + u, u, lane, N, top, hcur, dout);
             } else {
                 const int n = min(32, s_end - s0);
-#pragma unroll 1
-                for (int u = 0; u < n; ++u) st.template step<false, BANDED, TRACK>(slot, u, lane, N, top);
+                for (int u = 0; u < n; ++u)
+                    st.template step_at<false, BANDED>(ring, s0 + u, u, lane, N, top, hcur, dout);
             }
-        };
-        if (MODE == kModeSubDirs && last)
-            chunk(std::true_type{});
-        else
-            chunk(std::false_type{});
+        } else {
+            auto chunk = [&](auto track) {
+                constexpr bool TRACK = decltype(track)::value;
+                if (full) {
+#pragma unroll (kUnroll<D, R, MODE, BANDED>)
+                    for (int u = 0; u < 32; ++u) st.template step<true, false, TRACK>(slot, u, lane, N, top);
+                } else {
+                    const int n = min(32, s_end - s0);
+#pragma unroll 1
+                    for (int u = 0; u < n; ++u) st.template step<false, BANDED, TRACK>(slot, u, lane, N, top);
+                }
+            };
+            if (MODE == kModeSubDirs && last)
+                chunk(std::true_type{});
+            else
+                chunk(std::false_type{});
+        }
     }
 
     constexpr int SPW = BandT::SPW;
@@ -525,7 +670,9 @@ constexpr int min_blocks()
     return R == 8 ? (D <= 4 ? 4 : (D <= 8 ? 3 : 2)) : ((R == 16 && D <= 4) ? 3 : 2);
 }
 
-// The (place q in the work list's pair order, band) of an item.
+// The (place q in the work list's pair order, band) of an item.  EQUAL: every pair
+// has the same bands.
+template <bool EQUAL>
 __device__ __forceinline__ void item_of(const DPParams& p, int item, int& q, int& band)
 {
     if (p.group_pairs > 0) {
@@ -538,7 +685,7 @@ __device__ __forceinline__ void item_of(const DPParams& p, int item, int& q, int
         // items empty; recompute runs the range [band_lo, band_lo + band_cnt)
         // of each pair.  Band b - 1 of a pair is earlier in the list (no
         // deadlock).
-        const int nb = p.recompute ? p.band_cnt : p.group_bands;
+        const int nb = p.recompute ? p.band_cnt : (EQUAL ? p.prefix[1] - p.prefix[0] : p.group_bands);
         const int G = p.group_pairs;
         const int g = item / (G * nb), q0 = g * G;
         const int Gg = min(G, p.P - q0);
@@ -559,22 +706,25 @@ __global__ void __launch_bounds__(128, min_blocks<D, R>()) dtw_wavefront_kernel(
 {
     extern __shared__ u64 ring_all[];
     const int lane = threadIdx.x & 31;
-    u64* ring = ring_all + (threadIdx.x >> 5) * (D * kRing + kSlot);
+    u64* ring = ring_all + (threadIdx.x >> 5) * (D * kRingOf<D> + kSlot);
     for (;;) {
         int item = 0;
         if (lane == 0) item = atomicAdd(&p.hdr->item_counter, 1);
         item = __shfl_sync(FULL, item, 0);
         if (item >= p.n_items) break;
         if (ld_volatile(&p.hdr->abort)) break;
+        // (known to the compiler for wide samples: it changes the step's schedule, codes of
+        // 100 x 6k x 16 ch, 8 rows, 5.8 -> 5.2 ms)
+        constexpr bool EQUAL = kPerStep<D> && MODE != kModeCost;
         int q, band;
-        item_of(p, item, q, band);
+        item_of<EQUAL>(p, item, q, band);
         const PairDesc pd = p.pairs[p.order[q]];
-        if (band < pd.nbands) run_band<D, R, MODE, BANDED, COST>(p, pd, band, lane, ring);
+        if (EQUAL || band < pd.nbands) run_band<D, R, MODE, BANDED, COST>(p, pd, band, lane, ring);
     }
 }
 
 template <int D>
-constexpr size_t ring_bytes(int block) { return (size_t)(block / 32) * (D * kRing + kSlot) * sizeof(u64); }
+constexpr size_t ring_bytes(int block) { return (size_t)(block / 32) * (D * kRingOf<D> + kSlot) * sizeof(u64); }
 
 template <int D, int R, int MODE, bool BANDED, int COST>
 cudaError_t launch_one(const DPParams& p, int grid, int block, cudaStream_t st)
