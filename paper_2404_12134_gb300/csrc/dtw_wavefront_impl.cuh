@@ -104,12 +104,14 @@ __device__ __forceinline__ uint32_t ne_mask(float a, float b)
 // loads need no address arithmetic.
 constexpr int kRing = 164;
 __device__ __forceinline__ int ring_place(int s0) { return (s0 & 127) ? (s0 & 127) : 128; }
-// From seven channels on, but for nine, a step computes its own addresses (StepBand)
-// and the ring is the four chunks alone, without copies.
-template <int D>
-constexpr bool kPerStep = D > 6 && D != 9;
-template <int D>
-constexpr int kRingOf = kPerStep<D> ? 128 : kRing;
+// From seven channels on, but for nine, and for one channel's count at 16 rows, a step
+// computes its own addresses (StepBand) and the ring is the four chunks alone, without
+// copies.
+template <int D, int R, int MODE, int COST>
+constexpr bool kPerStep = (D > 6 && D != 9) ||
+                          (D == 1 && R == 16 && MODE == kModePlen && COST == kCostSqEuclid);
+template <int D, int R, int MODE, int COST>
+constexpr int kRingOf = kPerStep<D, R, MODE, COST> ? 128 : kRing;
 constexpr int kSlot = 4;     // u64 words after a warp's ring: its band's columns and the band
 
 
@@ -344,14 +346,15 @@ struct Band {
 // memory of two blocks 130 -> 170 KB of the SM's 256).  Wavefront, 300 pairs of 6k (100 at 16
 // channels), 16 rows, per chunk / per step in ms: 8 channels codes 8.5 / 7.7, 16
 // channels codes 10.9 / 7.0, cost + |pi| 16.5 / 9.0, l2 checkpointed 50 / 23.6, Sub-DTW
-// l2 28 / 13.4, 12 channels 28 / 23.4.  At nine channels: codes 8.4 / 9.4.
+// l2 28 / 13.4, 12 channels 28 / 23.4.  At nine channels: codes 8.4 / 9.4.  One channel,
+// cost + |pi|, 16 rows: 3.79 / 3.35, under a band of 0.4 3.46 / 3.34.
 template <int D, int R, int MODE, bool BANDED, int COST>
 struct StepBand : Band<D, R, MODE, BANDED, COST> {
     using B = Band<D, R, MODE, BANDED, COST>;
     using B::CODES; using B::W; using B::Q;
     using B::col; using B::dl; using B::cnt; using B::prev_up; using B::prev_upc; using B::topv; using B::topc;
     using B::half; using B::kk; using B::best; using B::bestj; using B::cost_pair;
-    static constexpr int RING = kRingOf<D>;
+    static constexpr int RING = kRingOf<D, R, MODE, COST>;
     bool track;
 
     __device__ __forceinline__ void load_column(const u64* ring, int jc, u64* yy)
@@ -456,9 +459,11 @@ struct StepBand : Band<D, R, MODE, BANDED, COST> {
 template <int D, int R, int MODE, bool BANDED, int COST>
 __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, int band, int lane, u64* ring)
 {
-    using BandT = std::conditional_t<kPerStep<D>, StepBand<D, R, MODE, BANDED, COST>, Band<D, R, MODE, BANDED, COST>>;
+    constexpr bool PER_STEP = kPerStep<D, R, MODE, COST>;
+    using BandT =
+        std::conditional_t<PER_STEP, StepBand<D, R, MODE, BANDED, COST>, Band<D, R, MODE, BANDED, COST>>;
     constexpr int BR = BandT::BR;
-    constexpr int RING = kRingOf<D>;
+    constexpr int RING = kRingOf<D, R, MODE, COST>;
     constexpr int W = BandT::W;
     const int M = pd.M, N = pd.N, d = p.d;
     const int i0 = band * BR + lane * R;
@@ -484,7 +489,7 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     st.topv = INF;
     st.topc = 0;
     st.half = 0u;
-    if constexpr (kPerStep<D>) st.track = MODE == kModeSubDirs && last;
+    if constexpr (PER_STEP) st.track = MODE == kModeSubDirs && last;
     st.kk = M - 1 - i0;
     st.best = INF;
     st.bestj = 0;
@@ -548,7 +553,7 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
             u64* row = ring + c * RING;
             const u64 v = pack2(ynext[c], ynext[c]);
             const int i = jj & 127;
-            if (kPerStep<D>) {
+            if (PER_STEP) {
                 row[i] = v;
                 continue;
             }
@@ -569,11 +574,11 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
     load_y(s_begin + lane + 64);
     if (!top) tnext = load_t(s_begin + lane);
     __syncwarp();
-    if constexpr (!kPerStep<D>) st.begin_chunk(ring, s_begin, lane, hcur, dout);
+    if constexpr (!PER_STEP) st.begin_chunk(ring, s_begin, lane, hcur, dout);
     {
         // local costs of the lane's first column (j = s_begin - lane)
         u64 yy[D];
-        if constexpr (kPerStep<D>)
+        if constexpr (PER_STEP)
             st.load_column(ring, s_begin - lane, yy);
         else
             st.load_samples(0, yy);
@@ -603,12 +608,12 @@ __device__ __forceinline__ void run_band(const DPParams& p, const PairDesc& pd, 
                 tnext = load_t(jj + 32);
             }
         }
-        if constexpr (!kPerStep<D>) st.begin_chunk(ring, s0, lane, hcur, dout);
+        if constexpr (!PER_STEP) st.begin_chunk(ring, s0, lane, hcur, dout);
         // every lane in the band's columns and inside the band all chunk long
         const bool full = BANDED ? (s0 - 31 >= jlo_b && s0 + 31 <= jhi_b &&
                                     __all_sync(FULL, s0 - lane >= full_lo && s0 + 31 - lane <= full_hi))
                                  : (s0 >= 31 && s0 + 32 <= N);
-        if constexpr (kPerStep<D>) {
+        if constexpr (PER_STEP) {
             if (full) {
 #pragma unroll 2
                 for (int u = 0; u < 32; ++u) st.template step_at<true>(ring, s0 + u, u, lane, N, top, hcur, dout);
@@ -706,7 +711,7 @@ __global__ void __launch_bounds__(128, min_blocks<D, R>()) dtw_wavefront_kernel(
 {
     extern __shared__ u64 ring_all[];
     const int lane = threadIdx.x & 31;
-    u64* ring = ring_all + (threadIdx.x >> 5) * (D * kRingOf<D> + kSlot);
+    u64* ring = ring_all + (threadIdx.x >> 5) * (D * kRingOf<D, R, MODE, COST> + kSlot);
     for (;;) {
         int item = 0;
         if (lane == 0) item = atomicAdd(&p.hdr->item_counter, 1);
@@ -715,7 +720,7 @@ __global__ void __launch_bounds__(128, min_blocks<D, R>()) dtw_wavefront_kernel(
         if (ld_volatile(&p.hdr->abort)) break;
         // (known to the compiler for wide samples: it changes the step's schedule, codes of
         // 100 x 6k x 16 ch, 8 rows, 5.8 -> 5.2 ms)
-        constexpr bool EQUAL = kPerStep<D> && MODE != kModeCost;
+        constexpr bool EQUAL = kPerStep<D, R, MODE, COST> && MODE != kModeCost;
         int q, band;
         item_of<EQUAL>(p, item, q, band);
         const PairDesc pd = p.pairs[p.order[q]];
@@ -723,13 +728,16 @@ __global__ void __launch_bounds__(128, min_blocks<D, R>()) dtw_wavefront_kernel(
     }
 }
 
-template <int D>
-constexpr size_t ring_bytes(int block) { return (size_t)(block / 32) * (D * kRingOf<D> + kSlot) * sizeof(u64); }
+template <int D, int R, int MODE, int COST>
+constexpr size_t ring_bytes(int block)
+{
+    return (size_t)(block / 32) * (D * kRingOf<D, R, MODE, COST> + kSlot) * sizeof(u64);
+}
 
 template <int D, int R, int MODE, bool BANDED, int COST>
 cudaError_t launch_one(const DPParams& p, int grid, int block, cudaStream_t st)
 {
-    const size_t smem = ring_bytes<D>(block);
+    const size_t smem = ring_bytes<D, R, MODE, COST>(block);
     cudaFuncSetAttribute(dtw_wavefront_kernel<D, R, MODE, BANDED, COST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     dtw_wavefront_kernel<D, R, MODE, BANDED, COST><<<grid, block, smem, st>>>(p);
@@ -740,7 +748,7 @@ template <int D, int R, int MODE, bool BANDED, int COST>
 int occ_one(int block)
 {
     int n = 0;
-    const size_t smem = ring_bytes<D>(block);
+    const size_t smem = ring_bytes<D, R, MODE, COST>(block);
     cudaFuncSetAttribute(dtw_wavefront_kernel<D, R, MODE, BANDED, COST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dtw_wavefront_kernel<D, R, MODE, BANDED, COST>, block, smem);
