@@ -54,14 +54,14 @@ constexpr RowTable kRowTable[] = {
          {{220, 198, 152}, {192, 190, 152}}, {}}},
     {6, {{{75, 72, 66}, {64, 63, 56}}, {{107, 108, 97}, {133, 116, 104}},
          {{203, 201, 199}, {250, 190, 199}}, {}}},
-    {8, {{{83, 79, 73}, {80, 81, 74}}, {{142, 127, 112}, {157, 146, 133}},
-         {{327, 237, 231}, {268, 285, 256}}, {}}},
+    {8, {{{83, 79, 73}, {80, 81, 74}}, {{139, 136, 121}, {160, 134, 126}},
+         {{284, 238, 223}, {254, 240, 262}}, {}}},
     {9, {{{83, 82, 77}, {86, 90, 81}}, {{133, 133, 116}, {155, 146, 146}},
          {{326, 326, 245}, {269, 296, 272}}, {}}},
-    {12, {{{97, 96, 88}, {99, 100, 102}}, {{160, 161, 149}, {196, 192, 187}},
-         {{602, 595, 486}, {406, 408, 365}}, {}}},
-    {16, {{{123, 123, 113}, {130, 133, 139}}, {{209, 201, 183}, {251, 243, 241}},
-         {{1287, 1000, 1021}, {1361, 901, 1255}}, {}}},
+    {12, {{{97, 96, 88}, {99, 100, 102}}, {{172, 175, 157}, {202, 185, 161}},
+         {{603, 584, 497}, {400, 395, 348}}, {}}},
+    {16, {{{123, 123, 113}, {130, 133, 139}}, {{210, 216, 197}, {248, 225, 208}},
+         {{928, 801, 846}, {697, 565, 580}}, {}}},
 };
 constexpr double kSchedulers = 4 * 152;
 
