@@ -449,7 +449,7 @@ def long_leg(api, torch, dev, barrier, iters: int = 2, cpu_sample: bool = True, 
     res["options"] = {"rows_per_thread": tuned.rows_per_thread, "warps_per_block": tuned.warps_per_block}
     for name, mode in (("stored", 0), ("checkpoint", 1)):
         opt = api.options(rows_per_thread=tuned.rows_per_thread, warps_per_block=tuned.warps_per_block,
-                          dir_mode=mode, ckpt_bands=16)
+                          rows_by_size=tuned.rows_by_size, dir_mode=mode, ckpt_bands=16)
         if ws is None:
             ws = api.Workspace(dev)
         B = B0.clone()
@@ -749,8 +749,7 @@ def small_dba_leg(api, torch, dev, barrier, cpu_sample: bool = True):
     b = synth.config_batch(0)
     gb = api.Batch.from_numpy(b.data, b.offsets, device=dev)
     ws = api.Workspace(dev)
-    # launch shape for this small batch (untimed; cached): 32 rows per lane
-    # give 2 bands per pair, fewer rows more and shorter bands
+    # launch shape for this small batch (untimed; cached)
     idx, _ = api.medoid(api.pairwise_dtw(gb, ws=ws))
     Bw = gb.data[int(b.offsets[int(idx)]):int(b.offsets[int(idx) + 1])].clone()
     dopt, _ = api.autotune(_abi.OP_DBA_ITERATE, Bw, gb, ws)
@@ -782,7 +781,8 @@ def small_dba_leg(api, torch, dev, barrier, cpu_sample: bool = True):
            "gcups": cells0 / (it_ms * 1e-3) / 1e9, "medoid_10_iterations_scores_s": total,
            "per_pair_align_s_per_iter": pp_ms * 1e-3, "device_status": api.read_status(ws.buf),
            "options": {"dba_rows_per_thread": dopt.rows_per_thread, "dba_warps_per_block": dopt.warps_per_block,
-                       "score_rows_per_thread": sopt.rows_per_thread,
+                       "dba_rows_by_size": dopt.rows_by_size, "score_rows_per_thread": sopt.rows_per_thread,
+                       "score_rows_by_size": sopt.rows_by_size,
                        "score_form": "codes + walk" if sopt.score_via_codes else "count inside the DP"}}
     if cpu_sample:
         # the oracle's inputs come from the generator only (its time does not

@@ -16,7 +16,9 @@
 // Measured (one pair, cost + |pi|): a step of 128 rows 62 ns at one channel, 83 at
 // nine, bands 66 steps apart; 1.1k x 1.1k x 1 ch 102 us against 121 with 8 rows per
 // lane and 265 with 32; Sub-DTW windows of 16k x 32k x 9 ch 6.35 -> 3.5 ms.  Bound
-// by dependent latencies: about 28 instructions a step at 3.3 cycles each.
+// by dependent latencies: a step's 128 cycles (one channel, 2.07 GHz) hold the shuffle
+// from the lane above and, one after the other down four rows, a minimum, an addition
+// and the count's selects, with one warp on a scheduler to issue them.
 #pragma once
 
 #include "dtw_wavefront_impl.cuh"

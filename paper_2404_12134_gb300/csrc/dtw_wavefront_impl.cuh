@@ -114,8 +114,10 @@ template <int D, int R, int MODE, int COST>
 constexpr int kRingOf = kPerStep<D, R, MODE, COST> ? 128 : kRing;
 constexpr int kSlot = 4;     // u64 words after a warp's ring: its band's columns and the band
 
-
-
+// Up to this many channels a code bit is the sign of m - v (an FMA-pipe subtraction
+// and a funnel shift), from there on a comparison to a mask (two ALU instructions and
+// their share of an OR): with six channels the FMA pipe is the fuller one (60 pairs
+// of 16k x 4 ch by sign 12.9 -> 10.2 ms; 200 of 25k x 6 ch 70.0 -> 83.5).
 constexpr int kSignD = 4;
 
 // Steps of the inner loop unrolled.  Four where a step is short (8 rows up to four
@@ -287,12 +289,10 @@ struct Band {
                         // the sign of m - v (0 when equal, also at +inf: that NaN is positive)
                         pl0 = __funnelshift_l(__float_as_uint(__fsub_rn(m, dg)), pl0, 1);
                         pl1 = __funnelshift_l(__float_as_uint(__fsub_rn(m, up)), pl1, 1);
-                    } else if (R < 32) {
+                    } else {
+                        static_assert(R < 32 || SIGNS, "32 rows' codes are taken by sign");
                         pl0 |= ne_mask(dg, m) & (1u << (R - 1 - k));
                         pl0 |= ne_mask(up, m) & (1u << ((2 * R - 1 - k) & 31));
-                    } else {
-                        pl0 |= ne_mask(dg, m) & (1u << (R - 1 - k));
-                        pl1 |= ne_mask(up, m) & (1u << (R - 1 - k));
                     }
                 } else if (MODE == kModePlen) {
                     const int cl = cnt[k];

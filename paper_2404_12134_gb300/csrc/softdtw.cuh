@@ -62,7 +62,12 @@ struct SoftParams {
 //   32 x 8.0k x 8 ch   4707 + 8189 / 5579 + 10828   (1,024)
 //   64 x 8.0k x 1 ch   4434 + 6567 / 5182 + 8450    (2,048)
 // Prototypes over kSoftFewM rows keep 8, so that a long batch's workspaces with
-// R kept and with column checkpoints (8 rows always) differ by R alone.
+// R kept and with column checkpoints (8 rows always) differ by R alone (store_pairs is
+// sized by it); their time is not the reason, 4 rows would be faster there too:
+//    8 x 10k x 1 ch    4000 + 3233 / 3414 + 3232      (320)
+//    8 x 10k x 6 ch    4404 + 7103 / 3917 + 5024      (320)
+//   16 x 10k x 3 ch    4515 + 5847 / 3898 + 5938      (640)
+//    4 x 12k x 8 ch    5508 + 8710 / 4588 + 7640      (188)
 constexpr int kSoftFewBands = 768;
 constexpr int64_t kSoftFewM = 8192;
 inline int soft_rows(int64_t M, int T)
